@@ -471,7 +471,7 @@ def evd_kernel_classes(stats, wl, peaks):
     # an emulated FP64 product issues 36 bf16 slice products per FP64 product
     emu_slice = 36 * tot("flops_update") if emu else 0
     cls = {
-        "pivot": dict(kernel="k_pivot / k_pivot_cluster", ms=tot("ms_pivot"),
+        "pivot": dict(kernel="k_pivot_pos", ms=tot("ms_pivot"),
                       launches=tot("pivot_launches"),
                       flops=tot("flops_fp64") - (0 if emu else tot("flops_update")) - tot("flops_refine"),
                       bound="alu", peak=FP64_PEAK_TFLOPS, peak_basis=FP64_BASIS),
@@ -552,7 +552,7 @@ def svd_kernel_classes(stats, wl, peaks):
     emu = wl.get("precision", 0) == 5 or wl.get("fp64_products", 0) == 1
     kernels = {"update": dict(kernel="k_gram + k_update_cols", ms=tot("ms_update"),
                               launches=tot("update_launches"), flops=tot("flops_update")),
-               "pivot": dict(kernel="k_pivot / k_pivot_cluster (Gram pivots)", ms=tot("ms_pivot"),
+               "pivot": dict(kernel="k_pivot_pos (Gram pivots)", ms=tot("ms_pivot"),
                              launches=tot("pivot_launches"),
                              flops=tot("flops_fp64") - (0 if emu else tot("flops_update"))
                              - tot("flops_precond"))}

@@ -23,22 +23,20 @@
  *     (outputs then hold the current iterate), <0 an error (JACOBI_ERR_* or
  *     -k for an invalid k-th argument);
  *   - the pivot solves of a step with few pairs run with a thread-block
- *     cluster of up to 8 CTAs per pair (chosen automatically); the
+ *     cluster of up to 16 CTAs per pair (chosen automatically); the
  *     environment variable JACOBI_PIVOT_CLUSTER=1 forces one CTA per pair,
- *     =2/4/8 that cluster size where it fits.
+ *     =2/4/8/16 that cluster size where it fits.
  *
  * Environment switches (read at each call; none is needed):
- *   JACOBI_PIVOT_CLUSTER=1|2|4|8   pivot cluster size (above);
+ *   JACOBI_PIVOT_CLUSTER=1|2|4|8|16   pivot cluster size (above);
  *   JACOBI_BATCHED_LARGE=blocked|cluster|l2   route of the batched EVD
  *                                  orders above the shared-memory size
  *                                  (default blocked);
  *   JACOBI_BATCHED_SVD=rowwise     the batched one-sided SVD with one Gram
  *                                  entry per thread instead of staged row
  *                                  tiles (same results bit for bit);
- *   JACOBI_PIVOT_SCHEDULE=split|fused  round schedule of the cluster pivot
- *                                  solves (default: fused for 2b > 128,
- *                                  split below; the same results bit for
- *                                  bit);
+ *   JACOBI_PIVOT_SCHEDULE=split|fused  accepted, no effect (the cluster
+ *                                  pivot solves have one round schedule);
  *   JACOBI_EMU_IMAGE=0             the emulated FP64 products slice their
  *                                  operands in every tile instead of once
  *                                  into an image (V per step in the update,

@@ -81,7 +81,7 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
     pa.gscratch = E.gscratch;
     pa.qrws = E.qrws;
     pa.cnt = E.cnt;
-    cudaError_t e = E.pcl > 1 ? launch_pivot_cluster(pa, E.pcl, E.qtab, cs) : launch_pivot(pa, cs);
+    cudaError_t e = launch_pivot(pa, E.pcl, cs);
     if (e != cudaSuccess) return e;
     if (mid && (e = cudaEventRecordWithFlags(mid, cs, cudaEventRecordExternal)) != cudaSuccess) return e;
     UpdateArgs ua{};
@@ -202,7 +202,6 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
         E.cnt = ws.get<DevCounters>(1);
         int* rank = ws.get<int>(n);
         E.pcl = choose_pivot_cluster(E.k, E.ord.dev_per_step);
-        E.qtab = E.pcl > 1 ? ws.get<unsigned>(128 * 127 / 2) : nullptr;
         if (p.pivot_order == 2) E.qrws = ws.get<double>((size_t)E.ord.max_pairs * E.b * E.k);
         if (p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1) {
             E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, E.k));
@@ -222,7 +221,6 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
         }
         E.balance = p.conv == JACOBI_CONV_REL;
         if (ws.failed) return JACOBI_ERR_ALLOC;
-        if (E.qtab && launch_quad_table(E.qtab, 128, s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (E.err && cudaMemsetAsync(E.err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(E.dpairs, E.ord.dev_pairs.data(), E.ord.dev_pairs.size() * sizeof(int),
                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -333,12 +331,10 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         int* rank = ws.get<int>(n);
         DevCounters* cnt = ws.get<DevCounters>(1);
         const int pcl = choose_pivot_cluster(k, ord.dev_per_step);
-        unsigned* qtab = pcl > 1 ? ws.get<unsigned>(128 * 127 / 2) : nullptr;
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
         int* err = emu ? ws.get<int>(1) : nullptr;
         if (ws.failed) return JACOBI_ERR_ALLOC;
-        if (qtab && launch_quad_table(qtab, 128, s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),
                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaMemsetAsync(cnt, 0, sizeof(DevCounters), s) != cudaSuccess ||
@@ -390,7 +386,7 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                     pa.gscratch = gscr;
                     pa.qrws = qrws;
                     pa.cnt = cnt;
-                    if ((pcl > 1 ? launch_pivot_cluster(pa, pcl, qtab, cs) : launch_pivot(pa, cs)) != cudaSuccess)
+                    if (launch_pivot(pa, pcl, cs) != cudaSuccess)
                         return false;
                     if (launch_max_into(relmax, nps, sweepmax, cs) != cudaSuccess) return false;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 2], cs, cudaEventRecordExternal) != cudaSuccess) return false;
@@ -730,7 +726,6 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
         E.dpairs = ws.get<int2>(E.ord.dev_pairs.size() / 2);
         E.cnt = ws.get<DevCounters>(1);
         E.pcl = choose_pivot_cluster(E.k, E.ord.dev_per_step);
-        E.qtab = E.pcl > 1 ? ws.get<unsigned>(128 * 127 / 2) : nullptr;
         if (p.pivot_order == 2) E.qrws = ws.get<double>((size_t)E.ord.max_pairs * E.b * E.k);
         if (p.precision == JACOBI_PREC_FP64_EMU || (p.precision == JACOBI_PREC_FP64 && p.fp64_products == 1)) {
             E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, E.k));
@@ -753,7 +748,6 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
         E.balance = p.conv == JACOBI_CONV_REL;
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (E.err && cudaMemsetAsync(E.err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
-        if (E.qtab && launch_quad_table(E.qtab, 128, s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(E.dpairs, E.ord.dev_pairs.data(), E.ord.dev_pairs.size() * sizeof(int),
                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaMemsetAsync(E.cnt, 0, sizeof(DevCounters), s) != cudaSuccess ||
@@ -820,13 +814,11 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         double* smax = ws.get<double>(1);
         DevCounters* cnt = ws.get<DevCounters>(1);
         const int pcl = choose_pivot_cluster(k, nps);
-        unsigned* qtab = pcl > 1 ? ws.get<unsigned>(128 * 127 / 2) : nullptr;
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
         int* err = emu ? ws.get<int>(1) : nullptr;
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (err && cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
-        if (qtab && launch_quad_table(qtab, 128, s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),
                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaMemsetAsync(cnt, 0, sizeof(DevCounters), s) != cudaSuccess ||
@@ -860,7 +852,7 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         pa.gscratch = gscr;
         pa.qrws = qrws;
         pa.cnt = cnt;
-        if ((pcl > 1 ? launch_pivot_cluster(pa, pcl, qtab, s) : launch_pivot(pa, s)) != cudaSuccess ||
+        if (launch_pivot(pa, pcl, s) != cudaSuccess ||
             launch_max_into(relmax, nps, smax, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
         ColUpdateArgs ca{};

@@ -33,7 +33,6 @@ constexpr double U32 = 5.9604644775390625e-08;  // 2^-24
 struct LowpState {
     int np, b, k, n_real;
     int pcl = 1;
-    const unsigned* qtab = nullptr;
     const Ordering* ord;
     const int2* dpairs;
     float* Aw[2];
@@ -75,7 +74,7 @@ cudaError_t launch_step32(const LowpState& L, int s, int cur, cudaStream_t cs, d
     pa.gscratch = L.gscratch;
     pa.qrws = L.qrws;
     pa.cnt = L.cnt;
-    cudaError_t e = L.pcl > 1 ? launch_pivot_cluster(pa, L.pcl, L.qtab, cs) : launch_pivot(pa, cs);
+    cudaError_t e = launch_pivot(pa, L.pcl, cs);
     if (e != cudaSuccess) return e;
     if (mid && (e = cudaEventRecordWithFlags(mid, cs, cudaEventRecordExternal)) != cudaSuccess) return e;
     TcUpdArgs ua{};
@@ -221,7 +220,6 @@ int syev_mixed(int n, double* A, int lda, double* w, double* Q, int ldq, const j
     E.cnt = ws.get<DevCounters>(1);
     int* rank = ws.get<int>(n);
     E.pcl = choose_pivot_cluster(k, E.ord.dev_per_step);
-    E.qtab = E.pcl > 1 ? ws.get<unsigned>(128 * 127 / 2) : nullptr;
     if (p.pivot_order == 2) E.qrws = ws.get<double>((size_t)E.ord.max_pairs * p.b * k);
     // FP32 state (low-precision sweeps); pivot scratch shared with E
     L.Aw[0] = ws.get<float>(np2);
@@ -257,7 +255,6 @@ int syev_mixed(int n, double* A, int lda, double* w, double* Q, int ldq, const j
     }
     if (ws.failed) return JACOBI_ERR_ALLOC;
     L.pcl = E.pcl;
-    L.qtab = E.qtab;
     L.dpairs = E.dpairs;
     L.Vb = E.Vb;
     L.rot = E.rot;
@@ -268,7 +265,6 @@ int syev_mixed(int n, double* A, int lda, double* w, double* Q, int ldq, const j
     L.result = E.result;
     L.cnt = E.cnt;
 
-    if (E.qtab && launch_quad_table(E.qtab, 128, s) != cudaSuccess) return JACOBI_ERR_CUDA;
     if (cudaMemcpyAsync(E.dpairs, E.ord.dev_pairs.data(), E.ord.dev_pairs.size() * sizeof(int),
                         cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemsetAsync(E.cnt, 0, sizeof(DevCounters), s) != cudaSuccess ||
@@ -492,10 +488,7 @@ extern "C" int jacobi_syev_step_lowp(int np, float* A, int lda, float* Q, int ld
     L.err = ws.get<int>(1);
     L.cnt = ws.get<DevCounters>(1);
     L.pcl = choose_pivot_cluster(k, ord.dev_per_step);
-    unsigned* qtab = L.pcl > 1 ? ws.get<unsigned>(128 * 127 / 2) : nullptr;
-    L.qtab = qtab;
     if (ws.failed) return JACOBI_ERR_ALLOC;
-    if (qtab && launch_quad_table(qtab, 128, s) != cudaSuccess) return JACOBI_ERR_CUDA;
     const size_t row = (size_t)np * sizeof(float);
     if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),
                         cudaMemcpyHostToDevice, s) != cudaSuccess ||

@@ -150,22 +150,18 @@ inline bool emu_image_wanted()
 
 // Cluster size for the pivot solves of a step with npairs pairs of order k:
 // automatic unless JACOBI_PIVOT_CLUSTER is set ("1" = one CTA per pair, a
-// power of two <= 8 = that size when it fits).
+// power of two <= 16 = that size when it fits).
 inline int choose_pivot_cluster(int k, int npairs)
 {
-    int dev = 0, sms = 0, smem = 0;
+    int dev = 0, smem = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    int C = pivot_cluster_size(k, npairs, sms, (size_t)smem);
     if (const char* env = getenv("JACOBI_PIVOT_CLUSTER")) {
         const int want = atoi(env);
-        if (want == 1) C = 1;
-        else if (want == 2 || want == 4 || want == 8) {
-            if (k % want == 0 && k / want >= 8 && pivot_cluster_smem(k, want) + 8192 <= (size_t)smem) C = want;
-        }
+        if (want == 1) return 1;
+        if ((want == 2 || want == 4 || want == 8 || want == 16) && pivot_pos_fits(k, want, (size_t)smem)) return want;
     }
-    return C;
+    return pivot_cluster_size(k, npairs, (size_t)smem);
 }
 
 inline int check_params(const jacobi_params& p)
@@ -203,7 +199,6 @@ struct EvdState {
     int np, b, k;
     int n_real;   // rows/columns >= n_real are zero padding
     int pcl = 1;  // pivot cluster size (1: one CTA per pair)
-    unsigned* qtab = nullptr;
     Ordering ord;
     int2* dpairs;
     double* Aw[2];

@@ -62,7 +62,7 @@ cudaError_t launch_offnorm(int np, const double* Aw, double* partial, unsigned i
 cudaError_t launch_offnorm_ld(int n, const double* A, int ld, double* partial, unsigned int* ticket,
                               double* result, bool want_rel, cudaStream_t s);
 
-// Pivot solves of one step (one CTA per pair): reads Ain's pivot blocks
+// Pivot solves of one step: reads Ain's pivot blocks
 // (EVD) or sums the Gram partials (SVD), runs the FP64 inner Jacobi, writes
 // V (and V^T) per pair, D into Aout's pivot blocks (EVD), the rotation count
 // per pair and, for the SVD, the pre-rotation max normalised off-diagonal.
@@ -86,18 +86,15 @@ struct PivotArgs {
     int max_sweeps;
     int order;                 // 1: sort eigenpairs descending over real rows
     int n_real;                // rows/columns >= n_real are zero padding
-    double* gscratch;          // k > 128: per-pair global scratch (packed A + V)
+    double* gscratch;          // k > 128 with one CTA per pair: per-pair global scratch (packed A + V)
     double* qrws;              // order == 2: per-pair QRCP scratch, b x k doubles each
     DevCounters* cnt;
 };
-cudaError_t launch_pivot(const PivotArgs& a, cudaStream_t s);
-// The same pivot solves with a cluster of C CTAs per pair (C from
-// pivot_cluster_size; C == 1 means: use launch_pivot).  qtab: quad table
-// for half = 128 (device, from launch_quad_table).
-int pivot_cluster_size(int k, int npairs, int sms, size_t smem_cap);
-size_t pivot_cluster_smem(int k, int C);
-cudaError_t launch_pivot_cluster(const PivotArgs& a, int C, const unsigned* qtab, cudaStream_t s);
-cudaError_t launch_quad_table(unsigned* qtab, int h, cudaStream_t s);
+// with C CTAs per pair (C from pivot_cluster_size, or 1)
+cudaError_t launch_pivot(const PivotArgs& a, int C, cudaStream_t s);
+cudaError_t launch_pivot_pos(const PivotArgs& a, int C, cudaStream_t s);   // k <= 128, or C > 1
+bool pivot_pos_fits(int k, int C, size_t smem_cap);
+int pivot_cluster_size(int k, int npairs, size_t smem_cap);
 size_t pivot_gscratch_doubles(int k);   // per pair, 0 when shared memory suffices
 
 // Update of one step (EVD): sandwich items A'_{P1P2} = V1^T A_{P1P2} V2 for

@@ -75,29 +75,74 @@ __device__ __forceinline__ bool rotation_wanted(T app, T aqq, T apq, T tol)
 }
 
 // ---------------------------------------------------------------- FP64 with few FP64 instructions
-// On this part FP64 runs at 1/64 of the FP32 rate, and a correctly rounded
-// FP64 division or square root is a chain of about ten dependent FP64
-// instructions; the textbook rotation has four divisions and two square
-// roots in series.  The FP64 overloads below take FP32 seeds (FP32 runs on
-// the fast pipe) and refine them with Newton's method in FP64:
-//   * t is the root of g(t) = apq t^2 + (aqq - app) t - apq with |t| <= 1
-//     (the same root the textbook formula picks); the FP32 seed comes from
-//     t = sgn(zeta) |2 apq| / (|d| + sqrt(d^2 + 4 apq^2)), d = aqq - app,
-//     evaluated on d and apq scaled by a power of two, and Newton steps
-//     t <- t - g(t) r on the scaled g use the seed's r ~ 1/g'(t) (each step
-//     squares the relative error, 2^-22 -> 2^-44 -> below 2^-53);
-//   * c = 1/sqrt(1 + t^2) from an FP32 reciprocal square root y0 and one
-//     second-order step y = y0 (1 + h/2 + 3h^2/8), h = 1 - x y0^2;
-//   * tau = s/(1 + c) with 1/(1 + c) from an FP32 reciprocal r0 and one
-//     second-order step r = r0 (1 + e + e^2), e = 1 - (1 + c) r0.
-// The results agree with the textbook ones to a few units in the last
-// place, and c^2 + s^2 = 1 to the same order, so the rotation applied in
-// Rutishauser's form stays orthogonal to working precision.
+// On this part FP64 runs at 1/64 of the FP32 rate: any FP64 instruction, a
+// conversion included, holds its warp for 64 cycles, while an FP32 or integer
+// one takes about 5.  The rotation choice is the serial chain of a solve, so
+// the FP64 overloads below do all they can outside the FP64 unit:
+//   * conversions between FP64 and FP32 by integer instructions on the bits;
+//   * t (the root of a t^2 + d t - a = 0 with |t| <= 1, d = aqq - app, a = apq,
+//     the textbook's choice), tau (t tau^2 + 2 tau - t = 0) and s (s (1 +
+//     tau^2) = 2 tau) each from an FP32 seed and one Newton step in pairs of
+//     floats (exact products by fma, error-free sums): 2^-42 relative;
+//   * then one Newton step in FP64 each: two FMAs for the residual, one for
+//     the step with the seed's FP32 reciprocal of the derivative, one addition
+//     to join the pair.
+// 13 FP64 instructions in place of about 40 with single FP32 seeds, two FP64
+// Newton steps and hardware conversions.  t is within 2u of the exact root,
+// tau within 4u, s within 6u of the exact root's, and, since s follows from the
+// computed tau, (1 - s tau)^2 + s^2 = 1 within u (measured over 2e7 triples):
+// the rotation applied in Rutishauser's or the three-shear form stays
+// orthogonal to working precision.
 __device__ __forceinline__ int f64_biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
-__device__ __forceinline__ void schur2(double app, double aqq, double apq, double& s, double& t, double& tau)
+__device__ __forceinline__ float rsqrt_seed(float x)
 {
-    const double d = rn_sub(aqq, app);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_seed(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// |x| 2^(sh - e), e its exponent: the leading 24 bits (truncated), and the next
+// 23; 0 below 2^-80.  sh <= 0.
+__device__ __forceinline__ float f64_lead(double x, int sh)
+{
+    const int hi = __double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    return sh < -80 ? 0.0f : __int_as_float(((sh + 127) << 23) | ((hi & 0xFFFFF) << 3) | (int)(lo >> 29));
+}
+__device__ __forceinline__ float f64_rest(double x, int sh)
+{
+    const int lo = __double2loint(x);
+    return sh < -80 ? 0.0f
+                    : (__int_as_float(0x4B000000 | ((lo & 0x1FFFFFFF) >> 6)) - 8388608.0f) *
+                          __int_as_float((sh + 81) << 23);
+}
+// f 2^e exactly (f a normal float or 0, the result normal)
+__device__ __forceinline__ double f64_of(float f, int e)
+{
+    const int b = __float_as_int(f), m = b & 0x7fffffff;
+    return m < 0x00800000 ? 0.0 : __hiloint2double((b & 0x80000000) | ((m >> 3) + ((896 + e) << 20)), b << 29);
+}
+// the nearest float (ties away), 0 below the normal range; |x| < 2^127
+__device__ __forceinline__ float f32_of(double x)
+{
+    const long long v = (__double_as_longlong(x) & 0x7fffffffffffffffll) + (1ll << 28);
+    const long long m = (v >> 29) - (896ll << 23);
+    return m < 0x00800000 ? 0.0f : __int_as_float((int)m | (__double2hiint(x) & 0x80000000));
+}
+__device__ __forceinline__ double f64_signed(double x, int sign_bit)
+{
+    return __hiloint2double(__double2hiint(x) | sign_bit, __double2loint(x));
+}
+
+// any finite triple, by FP32 seeds and FP64 Newton steps on scaled values
+__device__ __forceinline__ void schur2_wide(double d, double apq, double& s, double& t, double& tau)
+{
     // scale d and apq by 2^(1022 - E'), E' = clamp(max exponent, 2, 2044): the larger lands in [0.5, 4)
     int E = max(f64_biased_exp(d), f64_biased_exp(apq));
     E = min(max(E, 2), 2044);
@@ -130,14 +175,79 @@ __device__ __forceinline__ void schur2(double app, double aqq, double apq, doubl
     tau = s * fma(r0, fma(e, e, e), r0);
 }
 
-// |apq| > tol sqrt|app| sqrt|aqq| as apq^2 > tol^2 |app| |aqq| where every
-// operand lies in [2^-400, 2^400] (no overflow or underflow in the squares;
-// nonnegative doubles compare like their bit patterns), else the square-root
-// form.
+__device__ __forceinline__ void schur2(double app, double aqq, double apq, double& s, double& t, double& tau)
+{
+    const double d = rn_sub(aqq, app);
+    const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(apq), E = max(Ed, Ea);
+    if (E < 128 || E > 1900 || Ea + 60 < E) {   // (the float pairs need apq within 2^-60 of d)
+        schur2_wide(d, apq, s, t, tau);
+        return;
+    }
+    const bool dzero = (__double_as_longlong(d) << 1) == 0;
+    const int sgn = dzero ? 0 : (__double2hiint(d) ^ __double2hiint(apq)) & 0x80000000;   // sgn(zeta), sgn(0) = +1
+    const double aa = fabs(apq), dd = fabs(d);
+    const float ah = f64_lead(aa, Ea - E), al = f64_rest(aa, Ea - E), dh = f64_lead(dd, Ed - E), dl = f64_rest(dd, Ed - E);
+    const float A = 2.0f * ah, n = fmaf(dh, dh, A * A), rs = rsqrt_seed(n);
+    const float t0 = A * rcp_seed(fmaf(n, rs, dh));
+    float te;
+    {   // residual a (t0^2 - 1) + d t0; its derivative at the root is sqrt(d^2 + 4 a^2)
+        const float P = dh * t0, Pe = fmaf(dh, t0, -P), p = t0 * t0, pe = fmaf(t0, t0, -p), Q = ah * p, Qe = fmaf(ah, p, -Q);
+        const float s1 = __fsub_rn(P, ah), b1 = __fsub_rn(s1, P);
+        const float e1 = __fadd_rn(__fsub_rn(P, __fsub_rn(s1, b1)), __fsub_rn(-ah, b1));
+        const float s2 = __fadd_rn(s1, Q), b2 = __fsub_rn(s2, s1);
+        const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(Q, b2));
+        const float low = ((e1 + e2) + (Pe + Qe)) + (fmaf(dl, t0, -al) + fmaf(al, p, ah * pe));
+        te = -(s2 + low) * rs;
+    }
+    const double td = f64_of(t0, 0) + f64_of(te, 0);
+    const double ta = fma(-fma(fma(aa, td, dd), td, -aa), f64_of(rs, 1023 - E), td);
+    const float c0 = rsqrt_seed(fmaf(t0, t0, 1.0f));
+    const float u0 = t0 * c0 * rcp_seed(1.0f + c0), s0 = t0 * c0, ry = fmaf(0.5f, c0, 0.5f);
+    float ue, se;
+    {
+        const float P = 2.0f * u0, p = u0 * u0, pe = fmaf(u0, u0, -p), Q = t0 * p, Qe = fmaf(t0, p, -Q);
+        const float s1 = __fsub_rn(P, t0), b1 = __fsub_rn(s1, P);
+        const float e1 = __fadd_rn(__fsub_rn(P, __fsub_rn(s1, b1)), __fsub_rn(-t0, b1));
+        const float s2 = __fadd_rn(s1, Q), b2 = __fsub_rn(s2, s1);
+        const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(Q, b2));
+        const float low = ((e1 + e2) + Qe) + (fmaf(t0, pe, te * p) - te);
+        ue = -0.5f * c0 * (s2 + low);
+        const float R = s0 * p, Re = fmaf(s0, p, -R);
+        const float r1 = __fsub_rn(P, s0), c1 = __fsub_rn(r1, P);
+        const float f1 = __fadd_rn(__fsub_rn(P, __fsub_rn(r1, c1)), __fsub_rn(-s0, c1));
+        const float r2 = __fsub_rn(r1, R), c2 = __fsub_rn(r2, r1);
+        const float f2 = __fadd_rn(__fsub_rn(r1, __fsub_rn(r2, c2)), __fsub_rn(-R, c2));
+        const float lw = ((f1 + f2) - Re) + (2.0f * ue - s0 * fmaf(2.0f * u0, ue, pe));
+        se = (r2 + lw) * ry;
+    }
+    const double ud = f64_of(u0, 0) + f64_of(ue, 0);
+    const double ua = fma(-fma(fma(ta, ud, 2.0), ud, -ta), f64_of(0.5f * c0, 0), ud);
+    const double sd = f64_of(s0, 0) + f64_of(se, 0);
+    const double sa = fma(fma(-sd, fma(ua, ua, 1.0), ua + ua), f64_of(ry, 0), sd);
+    t = f64_signed(ta, sgn);
+    tau = f64_signed(ua, sgn);
+    s = f64_signed(sa, sgn);
+}
+
+// |apq| > tol sqrt|app| sqrt|aqq| as apq^2 > tol^2 |app| |aqq|, first on
+// the leading 24 bits in FP32 with the exponents apart (no FP64 instruction):
+// the truncations move either side by less than 2^-20, so only a ratio within
+// 2^-18 of 1 needs FP64.  There, where every operand lies in [2^-400, 2^400],
+// the squares can neither overflow nor underflow and nonnegative doubles
+// compare like their bit patterns; elsewhere the square-root form.
 __device__ __forceinline__ bool rotation_wanted(double app, double aqq, double apq, double tol)
 {
     if ((__double_as_longlong(apq) << 1) == 0) return false;
-    const int ep = f64_biased_exp(apq), e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq);
+    const int ep = f64_biased_exp(apq), e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq), et = f64_biased_exp(tol);
+    if (ep >= 1 && e1 >= 1 && e2 >= 1 && et >= 1) {
+        const int sh = e1 + e2 + 2 * et - 2 * ep - 2046;   // rhs / lhs in [2^(sh - 2), 2^(sh + 4))
+        if (sh > 8) return false;
+        if (sh < -8) return true;
+        const float fa = f64_lead(apq, 0), ft = f64_lead(tol, 0);
+        const float x = fa * fa;
+        const float y = ((ft * ft) * f64_lead(app, 0)) * (f64_lead(aqq, 0) * __int_as_float((sh + 127) << 23));
+        if (fabsf(x - y) > 3.8e-6f * x) return x > y;
+    }
     const bool safe = ep >= 623 && ep <= 1423 && e1 >= 623 && e1 <= 1423 && e2 >= 623 && e2 <= 1423;
     if (safe) {
         const double lhs = apq * apq, rhs = (tol * tol) * (fabs(app) * fabs(aqq));

@@ -4,13 +4,14 @@
 // the GPU), so every kernel here is shaped to issue as few FP64 operations as
 // possible; memory traffic is far below what HBM/L2 can move at that rate.
 //
-//   k_pivot      one CTA per pair: the 2b x 2b pivot of Algorithm 2 (line
+//   k_pivot      one CTA per pair for pivots that fit no shared memory (k >
+//                128 where no cluster fits either; all others are solved by
+//                k_pivot_pos): the 2b x 2b pivot of Algorithm 2 (line
 //                "diagonalise the subproblem"), solved by parallel-ordered
-//                scalar Jacobi (Algorithm 2 applied with b = 1) in FP64.  The
-//                symmetric pivot lives in shared memory in packed lower form;
-//                one round rotates every disjoint 2x2 "quad" from both sides
-//                (J_i^T X J_j), a third fewer operations than separate row and
-//                column passes.
+//                scalar Jacobi (Algorithm 2 applied with b = 1) in FP64, in
+//                packed lower form in global scratch; one round rotates every
+//                disjoint 2x2 "quad" from both sides (J_i^T X J_j), a third
+//                fewer operations than separate row and column passes.
 //   k_update_evd the block-row and block-column updates of Algorithm 2 for all
 //                pairs of a step, fused per pair-block: A'_{P1P2} =
 //                V_{P1}^T A_{P1P2} V_{P2} is computed once and written with its
@@ -219,17 +220,15 @@ size_t pivot_gscratch_doubles(int k) { return k <= 128 ? 0 : tri_pad(k) + (size_
 static size_t pivot_smem_bytes(int k)
 {
     const int half = k / 2, nq = half * (half - 1) / 2;
-    size_t small = (size_t)4 * half * sizeof(double) + (size_t)k * sizeof(double) +
-                   (size_t)3 * half * sizeof(int) + (size_t)nq * sizeof(unsigned) + 64;
-    if (k <= 128) small += (tri_pad(k) + (size_t)k * k) * sizeof(double);
-    return small;
+    return (size_t)4 * half * sizeof(double) + (size_t)k * sizeof(double) + (size_t)3 * half * sizeof(int) +
+           (size_t)nq * sizeof(unsigned) + 64;
 }
 
 template <bool V32> struct VType { using T = double; };
 template <> struct VType<true> { using T = float; };
 
 // V32: V accumulated in FP32 (in the first half of its k x k double region)
-template <bool SMEM, bool V32>
+template <bool V32>
 __global__ void __launch_bounds__(PIV_T) k_pivot(PivotArgs a)
 {
     using VT = typename VType<V32>::T;
@@ -240,17 +239,9 @@ __global__ void __launch_bounds__(PIV_T) k_pivot(PivotArgs a)
     const bool frozen = entry(a.pairs, e, I, J);
     const size_t ntp = tri_pad(k);
 
-    double *Ap, *tail;
-    VT* V;
-    if (SMEM) {
-        Ap = smem;
-        V = reinterpret_cast<VT*>(smem + ntp);
-        tail = smem + ntp + (size_t)k * k;
-    } else {
-        Ap = a.gscratch + (size_t)e * (ntp + (size_t)k * k);
-        V = reinterpret_cast<VT*>(Ap + ntp);
-        tail = smem;
-    }
+    double* Ap = a.gscratch + (size_t)e * (ntp + (size_t)k * k);
+    VT* V = reinterpret_cast<VT*>(Ap + ntp);
+    double* tail = smem;
     CoreSmem<double> cs;
     cs.tau = tail;
     cs.s = cs.tau + half;
@@ -394,12 +385,12 @@ __global__ void __launch_bounds__(PIV_T) k_pivot(PivotArgs a)
     }
 }
 
-cudaError_t launch_pivot(const PivotArgs& a, cudaStream_t s)
+cudaError_t launch_pivot(const PivotArgs& a, int C, cudaStream_t s)
 {
     if (a.npairs <= 0) return cudaSuccess;
+    if (a.k <= 128 || C > 1) return launch_pivot_pos(a, C, s);
     size_t smem = pivot_smem_bytes(a.k);
-    void (*kern)(PivotArgs) = a.k <= 128 ? (a.v32 ? k_pivot<true, true> : k_pivot<true, false>)
-                                         : (a.v32 ? k_pivot<false, true> : k_pivot<false, false>);
+    void (*kern)(PivotArgs) = a.v32 ? k_pivot<true> : k_pivot<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<a.npairs, PIV_T, smem, s>>>(a);

@@ -175,7 +175,7 @@ extern "C" int jacobi_syev_step_noalloc(int np, double* A, int lda, double* Q, i
     pa.n_real = np;
     pa.gscratch = gscr;
     pa.cnt = d_cnt;
-    if (launch_pivot(pa, s) != cudaSuccess) return JACOBI_ERR_CUDA;
+    if (launch_pivot(pa, 1, s) != cudaSuccess) return JACOBI_ERR_CUDA;
     UpdateArgs ua{};
     ua.Ain = Acur;
     ua.Aout = Anext;
