@@ -25,10 +25,10 @@
  *   - the pivot solves of a step with few pairs run with a thread-block
  *     cluster of up to 16 CTAs per pair (chosen automatically); the
  *     environment variable JACOBI_PIVOT_CLUSTER=1 forces one CTA per pair,
- *     =2/4/8/16 that cluster size where it fits.
+ *     =2 .. 16 that cluster size where it fits.
  *
  * Environment switches (read at each call; none is needed):
- *   JACOBI_PIVOT_CLUSTER=1|2|4|8|16   pivot cluster size (above);
+ *   JACOBI_PIVOT_CLUSTER=1..16     pivot cluster size (above);
  *   JACOBI_BATCHED_LARGE=blocked|cluster|l2   route of the batched EVD
  *                                  orders above the shared-memory size
  *                                  (default blocked);

@@ -149,8 +149,8 @@ inline bool emu_image_wanted()
 }
 
 // Cluster size for the pivot solves of a step with npairs pairs of order k:
-// automatic unless JACOBI_PIVOT_CLUSTER is set ("1" = one CTA per pair, a
-// power of two <= 16 = that size when it fits).
+// automatic unless JACOBI_PIVOT_CLUSTER is set ("1" = one CTA per pair,
+// up to "16" = that size when it fits).
 inline int choose_pivot_cluster(int k, int npairs)
 {
     int dev = 0, smem = 0;
@@ -159,7 +159,7 @@ inline int choose_pivot_cluster(int k, int npairs)
     if (const char* env = getenv("JACOBI_PIVOT_CLUSTER")) {
         const int want = atoi(env);
         if (want == 1) return 1;
-        if ((want == 2 || want == 4 || want == 8 || want == 16) && pivot_pos_fits(k, want, (size_t)smem)) return want;
+        if (want > 1 && pivot_pos_fits(k, want, (size_t)smem)) return want;
     }
     return pivot_cluster_size(k, npairs, (size_t)smem);
 }

@@ -128,7 +128,6 @@ __device__ __forceinline__ void shear2(T s, T tau, T& x, T& y)
     x = fma(-tau, y, u);
 }
 
-template <int N> struct PpInt { static constexpr int value = N; };
 __device__ __forceinline__ double f64_negate(double x)   // no FP64 instruction
 {
     return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
@@ -155,7 +154,7 @@ __host__ __device__ inline PpSmem pp_smem(int k, int C, bool v32)
     const int h = k / 2;
     PpSmem s;
     s.buf = 4 * pp_chunk(k, C) + ((h + 1) & ~1);   // the quads' entries, then the pairs' own
-    const int vel = (k / C) * k;
+    const int vel = (k + C - 1) / C * k;
     const int vd = ((v32 ? (vel + 1) / 2 : vel) + 1) / 2 * 2;
     const int rest = vd + 20 * h + k + (v32 ? 2 * h : 0);
     s.two = (size_t)(2 * s.buf + rest) * 8 + (size_t)(2 * k + 2 * h) * sizeof(int) <= PP_SMEM_MAX;
@@ -182,7 +181,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     const int e0 = blockIdx.x / C, tid = threadIdx.x, nt = blockDim.x;
     const int k = a.k, b = a.b, h = k >> 1, nr = k - 1, NQ = pp_quads(k), chunk = pp_chunk(k, C);
     const int q_lo = min(NQ, r * chunk), nq = min(NQ, q_lo + chunk) - q_lo;
-    const int rows = k / C, r_lo = r * rows;
+    const int r_lo = r * k / C, rows = (r + 1) * k / C - r_lo;   // of V
     const PpSmem L = pp_smem(k, C, V32);
     // quads by entry [TT TB BT BB][chunk], then the pairs' own entries [h]; round
     // g reads buffer g & 1 and writes the other (or both are one)
@@ -350,22 +349,27 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
             if (cnt == 0) break;
         }
     };
-    // this CTA's rows of V by the round, by warp wi of NW: a lane is a row (and
-    // with fewer than 32 rows, the warp takes several pairs at a time)
-    const int vpw = rows < 32 ? 32 / rows : 1, vsub = rows < 32 ? (tid & 31) / rows : 0;
-    const int vrow = rows < 32 ? (tid & 31) - vsub * rows : tid & 31;
-    auto rotate_v = [&](int so, int rd, int wi, auto nw) {
-        constexpr int NW = decltype(nw)::value, U = 4;
-        if (vsub >= vpw) return;
-        const int step = NW * vpw;
-        for (int e = wi * vpw + vsub; e < h; e += U * step) {
+    // this CTA's rows of V by the round, by thread vt of VN.  Whole warps of
+    // rows: a warp takes pairs, a lane a row; else the (pair, row) items dealt
+    // to the threads in order.
+    const int vt = role == 2 ? tid - (nt - AT) : tid;
+    constexpr int VN = V32 ? (AT > 0 ? AT : 32) : NB;
+    const bool vwarp = rows % 32 == 0;
+    const int ve0 = vwarp ? vt >> 5 : vt / rows, vi0 = vwarp ? vt & 31 : vt - ve0 * rows;
+    const int vde = vwarp ? VN / 32 : VN / rows, vdi = vwarp ? 0 : VN - vde * rows;
+    auto rotate_v = [&](int so, int rd) {
+        constexpr int U = 4;
+        int e = ve0, i = vi0;
+        while (e < h) {
             int ot[U], ob[U];
             VT ps[U], pu[U];
+            bool on[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int f = min(e + u * step, h - 1);
-                ot[u] = rows * pp_index(f, rd, nr) + vrow;
-                ob[u] = rows * pp_index(k - 1 - f, rd, nr) + vrow;
+                on[u] = e < h;
+                const int f = min(e, h - 1);
+                ot[u] = rows * pp_index(f, rd, nr) + i;
+                ob[u] = rows * pp_index(k - 1 - f, rd, nr) + i;
                 if constexpr (V32) {
                     const float2 p = par32[so + f];
                     ps[u] = p.x;
@@ -375,30 +379,35 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                     ps[u] = p.x;
                     pu[u] = p.y;
                 }
+                e += vde;
+                i += vdi;
+                if (i >= rows) {
+                    i -= rows;
+                    ++e;
+                }
             }
-            for (int i = 0; i + vrow < rows; i += 32) {
+            for (int o = 0; o < (vwarp ? rows : 1); o += 32) {
                 VT xt[U], xb[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (e + u * step < h) {
-                        xt[u] = Vl[ot[u] + i];
-                        xb[u] = Vl[ob[u] + i];
+                    if (on[u]) {
+                        xt[u] = Vl[ot[u] + o];
+                        xb[u] = Vl[ob[u] + o];
                     }
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (e + u * step < h) {
+                    if (on[u]) {
                         shear2(ps[u], pu[u], xt[u], xb[u]);
-                        Vl[ot[u] + i] = xt[u];
-                        Vl[ob[u] + i] = xb[u];
+                        Vl[ot[u] + o] = xt[u];
+                        Vl[ob[u] + o] = xb[u];
                     }
             }
         }
     };
     // the diagonal, carried as hi + lo by one thread per entry (ld: its number
     // among this CTA's): the round's rotation applied, sent to the next position
-    const int dl_ = role == 2 ? tid - (nt - AT) : tid;
-    const bool dcar = role == (kAuxDiag ? 2 : 0) && (dl_ >> 1) < s_nce;
-    const int dside = dl_ & 1, de = dcar ? s_ce[dl_ >> 1] : 0;
+    const bool dcar = role == (kAuxDiag ? 2 : 0) && (vt >> 1) < s_nce;
+    const int dside = vt & 1, de = dcar ? s_ce[vt >> 1] : 0;
     int dg_to = 0, dg_rank = 0;
     if (dcar) {
         int t1 = dside, e1 = de;
@@ -499,7 +508,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                 }
             }
             if constexpr (!kAuxDiag) carry_diag(g);
-            if constexpr (!V32) rotate_v(so, rd, tid >> 5, PpInt<NB / 32>{});
+            if constexpr (!V32) rotate_v(so, rd);
         });
     } else if (role == 1) {
         const int cl = tid - NB, lead = cl & 1;            // lead: 0 the top's lane, 1 the bottom's
@@ -513,13 +522,19 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
             cslot = pp_qid(ci, cj, h) - q_lo + lead * chunk;
             pvd = place(0, ce, 1, ce);
         }
+        int nrot = 0;                                      // rotations this lane chose for the sweep
+        auto flush = [&](int sw) {
+            const int n = __reduce_add_sync(0xffffffffu, nrot);
+            if (n && (tid & 31) == 0) atomicAdd(&cnt0[sw & 3], n);
+            nrot = 0;
+        };
         int t1 = lead, e1 = ce;                            // where this lane's index goes
         pp_next(t1, e1, h);
         const int dgd = t1 * h + e1, dgr = s_own[e1];
         // the rotation of round g for the pair's entry av and this lane's
         // diagonal entry: parameters to every CTA, and the change of the
         // diagonal to the lanes that hold its next position
-        auto choose = [&](int g, int sweep, int rd, double av, double dv) {
+        auto choose = [&](int g, int rd, double av, double dv) {
             const double dother = __shfl_xor_sync(0xffffffffu, dv, 1);
             const double app = lead ? dother : dv, aqq = lead ? dv : dother;
             const bool on = mine && rotation_wanted(app, aqq, av, tol);
@@ -555,10 +570,9 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                 else pp_st2(pp_mapa((uint32_t)__cvta_generic_to_shared(d), dgr), tl, al);
                 pv = on ? 0.0 : av;
             }
-            const unsigned m = __ballot_sync(0xffffffffu, on && lead == 0);
-            if (m && (tid & 31) == 0) atomicAdd(&cnt0[sweep & 3], __popc(m));
+            nrot += on && lead == 0;
         };
-        if (max_sweeps > 0) choose(0, 0, 0, mine ? psm[pv0 + ce] : 0.0, mine ? fin[lead ? k - 1 - ce : ce] : 0.0);
+        if (max_sweeps > 0) choose(0, 0, mine ? psm[pv0 + ce] : 0.0, mine ? fin[lead ? k - 1 - ce : ce] : 0.0);
         rounds([&](int g, int sw, int rd, bool last) {
             const int so = (g & 1) * h, from = (g & 1) * flip, to = flip - from;
             const double* st = psm + from;
@@ -586,8 +600,10 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                     // column: pair cj's top, or its bottom for the last pair
                     av = ce == h - 1 ? yb : yt;
                 }
-                const bool wrap = rd + 1 == nr;
-                choose(g + 1, wrap ? sw + 1 : sw, wrap ? 0 : rd + 1, av, d.x + fma(c.x, c.y, d.y));
+                if (rd + 1 == nr) flush(sw);
+                choose(g + 1, rd + 1 == nr ? 0 : rd + 1, av, d.x + fma(c.x, c.y, d.y));
+            } else {
+                flush(sw);
             }
             may_store();
             if (mine && lead == 0) {
@@ -599,7 +615,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
         rounds([&](int g, int, int rd, bool) {
             loaded();
             if constexpr (kAuxDiag) carry_diag(g);
-            if constexpr (V32) rotate_v((g & 1) * h, rd, (tid - (nt - AT)) >> 5, PpInt<(AT > 0 ? AT : 32) / 32>{});
+            if constexpr (V32) rotate_v((g & 1) * h, rd);
             may_store();
         });
     }
@@ -774,10 +790,10 @@ cudaError_t pp_config(const PpLaunch& l, int C, int npairs, cudaLaunchAttribute*
 
 bool pivot_pos_fits(int k, int C, size_t smem_cap)
 {
-    return C <= PP_MAXC && (C == 1 || (k % C == 0 && k / C >= 8)) && pp_smem(k, C, false).bytes + PP_STATIC <= smem_cap;
+    return C <= PP_MAXC && (C == 1 || k / C >= 8) && pp_smem(k, C, false).bytes + PP_STATIC <= smem_cap;
 }
 
-// Cluster size for a step with npairs pairs: the largest power of two C whose
+// Cluster size for a step with npairs pairs: the largest C whose
 // clusters can all run at once (asked of the runtime: a GPU part holds whole
 // clusters only, so npairs * C <= SMs is not enough) and that still pays, or 1.
 // A round's FP64 work per CTA shrinks with C while the rotation choice and the
@@ -791,8 +807,8 @@ int pivot_cluster_size(int k, int npairs, size_t smem_cap)
 {
     const int cmax = k <= 32 ? 1 : (k <= 64 ? 4 : (k <= 96 ? 8 : PP_MAXC));
     int least = 2;   // above k = 128, several waves of the smallest clusters beat one CTA on global scratch
-    while (least <= PP_MAXC && !pivot_pos_fits(k, least, smem_cap)) least *= 2;
-    for (int C = cmax; C > 1; C /= 2) {
+    while (least <= PP_MAXC && !pivot_pos_fits(k, least, smem_cap)) ++least;
+    for (int C = cmax; C > 1; --C) {
         if (!pivot_pos_fits(k, C, smem_cap)) continue;
         cudaLaunchAttribute attr[1];
         cudaLaunchConfig_t cfg = {};
