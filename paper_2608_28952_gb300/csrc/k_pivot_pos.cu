@@ -20,9 +20,13 @@
 // per ~18 cycles for the whole SM, and one per 64 cycles for any one warp, so
 // four warps with independent work fill it and more only queue in front of
 // the serial chain below):
-//   * 4 bulk warps: each thread owns up to QPT quads: loads them all, rotates
-//     them in registers by round g, stores the results at their next
-//     positions, then rotates this CTA's rows of V;
+//   * 4 bulk warps (8 for the largest pivots): each thread owns up to QPT quads:
+//     loads them all, rotates them in registers by round g, stores the results
+//     at their next positions;
+//   * auxiliary warps: this CTA's rows of V, and the diagonal (hi + lo) by the
+//     rotations already chosen (where V's rotation would only get in the way
+//     of the choice, or has no warps of its own, the bulk warps do it after
+//     their quads);
 //   * chain warps, two lanes per pair of round g + 1: that pair's entry is one
 //     entry of one quad of round g (BT of quad (e - 1, e + 1); TT of (0, 1)
 //     and BB of (k/2 - 2, k/2 - 1) at the ends), so a pair of lanes rotates
@@ -30,11 +34,10 @@
 //     at its position, chooses round g + 1's rotation, sends the parameters
 //     to every CTA and the diagonal after that rotation to the lanes that
 //     need it next;
-//   * V in FP32 (a transform that only feeds the split low-precision
-//     products): 2 warps of their own, off the FP64 unit.
-// Two cluster barriers per round: "every quad of round g is in registers"
-// (stores may begin; its wait is hidden behind the rotations) and "round g is
-// stored, round g + 1's parameters are there".
+// One cluster barrier per round ("round g is stored, round g + 1's parameters
+// are there") with two buffers of the quads; where shared memory holds only
+// one, a second one ("every quad of round g is in registers") whose wait is
+// hidden behind the rotations.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <algorithm>
@@ -174,6 +177,12 @@ template <int NB, int QPT, int CH, int AT, bool V32>
 __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int C)
 {
     constexpr bool kAuxDiag = AT >= CH;   // the auxiliary threads carry the diagonal (else the first bulk threads)
+    // and rotate V: an FP32 one always; an FP64 one (as much work as the quads)
+    // where the FP64 unit bounds the round, not where the rotation choice does
+    // and would wait behind four more FP64 warps (one quad per bulk thread;
+    // measured: k = 32 78 us with V after the quads, 82 us beside them; k = 128
+    // with 16 pairs 613 and 520)
+    constexpr bool kAuxV = V32 || (AT > 0 && QPT > 1);
     using VT = typename PpV<V32>::T;
     extern __shared__ __align__(16) double psm[];
     cg::cluster_group cluster = cg::this_cluster();
@@ -353,7 +362,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // rows: a warp takes pairs, a lane a row; else the (pair, row) items dealt
     // to the threads in order.
     const int vt = role == 2 ? tid - (nt - AT) : tid;
-    constexpr int VN = V32 ? (AT > 0 ? AT : 32) : NB;
+    constexpr int VN = kAuxV ? AT : NB;
     const bool vwarp = rows % 32 == 0;
     const int ve0 = vwarp ? vt >> 5 : vt / rows, vi0 = vwarp ? vt & 31 : vt - ve0 * rows;
     const int vde = vwarp ? VN / 32 : VN / rows, vdi = vwarp ? 0 : VN - vde * rows;
@@ -454,12 +463,18 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
             dst[2 * u] = place(0, i, 0, j) | (place(0, i, 1, j) << 16);
             dst[2 * u + 1] = place(1, i, 0, j) | (place(1, i, 1, j) << 16);
         }
-        bool local = true;   // all of this thread's entries stay in this CTA
+        unsigned local = 0;   // bit u: all of quad u's entries stay in this CTA
 #pragma unroll
-        for (int u = 0; u < QPT; ++u)
-            if (tid + u * NB < nq)
+        for (int u = 0; u < QPT; ++u) {
+            bool l = true;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) local &= (int)(((dst[2 * u + (t >> 1)] >> (16 * (t & 1))) & 0xffffu) >> sh) == r;
+            for (int t = 0; t < 4; ++t) l &= (int)(((dst[2 * u + (t >> 1)] >> (16 * (t & 1))) & 0xffffu) >> sh) == r;
+            if (l) {              // (and then without the rank)
+                local |= 1u << u;
+                dst[2 * u] &= smask | (smask << 16);
+                dst[2 * u + 1] &= smask | (smask << 16);
+            }
+        }
         rounds([&](int g, int, int rd, bool) {
             const int so = (g & 1) * h, from = (g & 1) * flip, to = flip - from;
             const double* st = psm + from;
@@ -484,31 +499,27 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                 }
             }
             may_store();
-            if (local) {
-                double* sn = psm + to;
-                const uint32_t m = smask;
+            double* sn = psm + to;
 #pragma unroll
-                for (int u = 0; u < QPT; ++u) {
-                    if (tid + u * NB < nq) {
-                        sn[dst[2 * u] & m] = x[u][0];
-                        sn[(dst[2 * u] >> 16) & m] = x[u][1];
-                        sn[dst[2 * u + 1] & m] = x[u][2];
-                        sn[(dst[2 * u + 1] >> 16) & m] = x[u][3];
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < QPT; ++u) {
-                    if (tid + u * NB < nq) {
-                        put(to, dst[2 * u] & 0xffffu, x[u][0]);
-                        put(to, dst[2 * u] >> 16, x[u][1]);
-                        put(to, dst[2 * u + 1] & 0xffffu, x[u][2]);
-                        put(to, dst[2 * u + 1] >> 16, x[u][3]);
+            for (int u = 0; u < QPT; ++u) {
+                if (tid + u * NB < nq) {
+                    const uint32_t d0 = dst[2 * u] & 0xffffu, d1 = dst[2 * u] >> 16;
+                    const uint32_t d2 = dst[2 * u + 1] & 0xffffu, d3 = dst[2 * u + 1] >> 16;
+                    if ((local >> u) & 1) {
+                        sn[d0] = x[u][0];
+                        sn[d1] = x[u][1];
+                        sn[d2] = x[u][2];
+                        sn[d3] = x[u][3];
+                    } else {
+                        put(to, d0, x[u][0]);
+                        put(to, d1, x[u][1]);
+                        put(to, d2, x[u][2]);
+                        put(to, d3, x[u][3]);
                     }
                 }
             }
             if constexpr (!kAuxDiag) carry_diag(g);
-            if constexpr (!V32) rotate_v(so, rd);
+            if constexpr (!kAuxV) rotate_v(so, rd);
         });
     } else if (role == 1) {
         const int cl = tid - NB, lead = cl & 1;            // lead: 0 the top's lane, 1 the bottom's
@@ -615,7 +626,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
         rounds([&](int g, int, int rd, bool) {
             loaded();
             if constexpr (kAuxDiag) carry_diag(g);
-            if constexpr (V32) rotate_v((g & 1) * h, rd);
+            if constexpr (kAuxV) rotate_v((g & 1) * h, rd);
             may_store();
         });
     }
