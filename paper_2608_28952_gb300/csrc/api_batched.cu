@@ -12,6 +12,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -128,6 +129,8 @@ Shape evd_default(int esize, bool vec)
 }  // namespace
 
 // ============================================================================ plan
+constexpr int kBatchedSides = 5;   // the blocked method and clusters of 2, 4, 8, 16
+
 struct jacobi_plan {
     int kind;            // 0 syev, 1 gesvd
     int precision;       // JACOBI_PREC_FP64 / FP32
@@ -156,6 +159,9 @@ struct jacobi_plan {
     size_t blk_slot = 0;
     int blk_grid = 0;
     float last_ms = 0.f;
+    // symmetric EVD: side streams for the groups of a launch, and their events
+    cudaStream_t side[kBatchedSides] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[kBatchedSides] = {};
 };
 
 namespace {
@@ -164,6 +170,75 @@ size_t max_slot_elems(int kmax, bool vec)
 {
     return batched_tri_pad(kmax) + (vec ? (size_t)kmax * kmax : 0);
 }
+
+// CTAs per matrix for the blocked method on the `nb` largest matrices of the
+// list: one while the batch fills the GPU by itself, more when its longest
+// matrices on one CTA each would outlast the rest.  The longest-first queue is
+// played through for each C with the times measured on GB300 (C = 1 / 2 / 4 /
+// 8, n = 352: FP64 488 / 248 / 150 / 101 ms, FP32 29.3 / 21.9 / 18.2 / 17.0 ms;
+// n = 512: FP64 1463 / 746 / 400 / 240 ms, FP32 73.5 / 46.9 / 35.0 / 30.0 ms:
+// n^2.93 and n^2.45 on one CTA, and the smaller order's gain from C).  200
+// matrices of order 8..512: FP64 1756 -> 734 ms with the groups side by side,
+// FP32 87 -> 55 ms.
+template <typename T>
+int blk_cluster(const jacobi_plan* pl, const std::vector<int>& h_list, int nb)
+{
+    constexpr bool f64 = sizeof(T) == 8;
+    const double gain[4] = {1.0, f64 ? 1.96 : 1.34, f64 ? 3.25 : 1.61, f64 ? 4.85 : 1.72};
+    double best = 0.0;
+    int pick = 1;
+    for (int l = 0; l < 4; ++l) {
+        const int C = 1 << l;
+        std::priority_queue<double, std::vector<double>, std::greater<double>> ends;   // when each cluster is free
+        double last = 0.0;
+        for (int i = 0; i < nb; ++i) {
+            double t = pow((double)pl->h_n[h_list[i]], f64 ? 2.93 : 2.45) / gain[l];
+            if ((int)ends.size() == std::max(1, pl->blk_grid / C)) {
+                t += ends.top();
+                ends.pop();
+            }
+            ends.push(t);
+            last = std::max(last, t);
+        }
+        if (l == 0 || last < 0.9 * best) {
+            best = last;
+            pick = C;
+        }
+    }
+    return pick;
+}
+
+// Side streams of one launch of the batch: what runs beside the caller's
+// stream starts after what is on it now, and the stream waits for all of it.
+struct Fork {
+    jacobi_plan* pl;
+    cudaStream_t s;
+    int used = 0;
+    bool ok = true;
+    Fork(jacobi_plan* p, cudaStream_t st) : pl(p), s(st) {}
+    // a side stream (made when first wanted, kept by the plan); s when there is none left
+    cudaStream_t next()
+    {
+        if (!ok || used == kBatchedSides) return s;
+        if (!pl->ev_fork) ok = cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+        if (ok && used == 0) ok = cudaEventRecord(pl->ev_fork, s) == cudaSuccess;
+        if (ok && !pl->side[used]) {
+            int lo = 0, hi = 0;
+            ok = cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
+                 cudaStreamCreateWithPriority(&pl->side[used], cudaStreamNonBlocking, used == 0 ? hi : lo) == cudaSuccess;
+        }
+        if (ok && !pl->ev_join[used]) ok = cudaEventCreateWithFlags(&pl->ev_join[used], cudaEventDisableTiming) == cudaSuccess;
+        ok = ok && cudaStreamWaitEvent(pl->side[used], pl->ev_fork, 0) == cudaSuccess;
+        return ok ? pl->side[used++] : s;
+    }
+    cudaError_t join()
+    {
+        for (int i = 0; i < used; ++i)
+            ok = cudaEventRecord(pl->ev_join[i], pl->side[i]) == cudaSuccess &&
+                 cudaStreamWaitEvent(s, pl->ev_join[i], 0) == cudaSuccess && ok;
+        return ok ? cudaSuccess : cudaErrorUnknown;
+    }
+};
 
 // Launch the batch (or the sub-list `h_list` / `d_list`, matrix indices in
 // longest-first order): EVD matrices above the shared-memory size go to the
@@ -177,6 +252,10 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
     if (e != cudaSuccess) return e;
     const int B = pl->batch, count = (int)h_list.size();
     if (pl->kind == 0) {
+        // The groups below are independent: each goes to a stream of its own (the
+        // largest orders on the one with the highest priority), so that one group's last matrices
+        // do not leave the GPU idle before the next group starts.
+        Fork fork(pl, s);
         BatchedEvdArgs<T> a{};
         a.n = pl->d_n;
         a.A = (T* const*)pl->d_ptrs;
@@ -209,8 +288,9 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
                 if (k <= sh.smem_kmax || k <= blk_min) break;
                 ++nb;
             }
-            if ((e = launch_batched_evd_blocked<T>(a, d_list, nb, pl->d_queue + 1, (T*)pl->d_blk, pl->blk_slot,
-                                                   pl->blk_grid, s)) != cudaSuccess)
+            if (nb > 0 && (e = launch_batched_evd_blocked<T>(a, d_list, nb, pl->d_queue + 1, (T*)pl->d_blk, pl->blk_slot,
+                                                             pl->blk_grid, blk_cluster<T>(pl, h_list, nb), fork.next())) !=
+                              cudaSuccess)
                 return e;
             nl = nb;
             while (nl < count) {
@@ -228,7 +308,7 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
                     ++j;
                 }
                 const int kmax = (n0 + C - 1) / C * C;
-                if ((e = launch_batched_evd_cluster<T>(a, d_list + i, j - i, kmax, C, s)) != cudaSuccess) return e;
+                if ((e = launch_batched_evd_cluster<T>(a, d_list + i, j - i, kmax, C, fork.next())) != cudaSuccess) return e;
                 i = j;
             }
         } else if (pl->large_mode == 1) {
@@ -251,14 +331,14 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
                     ++j;
                 }
                 const int kmax = (n0 + C - 1) / C * C;
-                if ((e = launch_batched_evd_cluster<T>(a, d_list + i, j - i, kmax, C, s)) != cudaSuccess) return e;
+                if ((e = launch_batched_evd_cluster<T>(a, d_list + i, j - i, kmax, C, fork.next())) != cudaSuccess) return e;
                 i = j;
             }
         }
         a.batch = count - nl;
         a.order = d_list + nl;
-        if (a.batch == 0) return cudaSuccess;
-        return launch_batched_evd<T>(a, grid, sh.threads, s);
+        if (a.batch > 0 && (e = launch_batched_evd<T>(a, grid, sh.threads, s)) != cudaSuccess) return e;
+        return fork.join();
     }
     BatchedSvdArgs<T> a{};
     a.batch = count;
@@ -587,6 +667,11 @@ extern "C" void jacobi_plan_destroy(jacobi_plan* pl)
 {
     if (!pl) return;
     if (pl->exec) cudaGraphExecDestroy(pl->exec);
+    for (int i = 0; i < kBatchedSides; ++i) {
+        if (pl->ev_join[i]) cudaEventDestroy(pl->ev_join[i]);
+        if (pl->side[i]) cudaStreamDestroy(pl->side[i]);
+    }
+    if (pl->ev_fork) cudaEventDestroy(pl->ev_fork);
     cudaFree(pl->d_order);
     cudaFree(pl->d_m);
     cudaFree(pl->d_n);

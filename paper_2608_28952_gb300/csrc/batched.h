@@ -85,6 +85,6 @@ template <typename T>
 size_t batched_blocked_slot_elems(int nmax);
 template <typename T>
 cudaError_t launch_batched_evd_blocked(const BatchedEvdArgs<T>& a, const int* list, int count, unsigned* queue,
-                                       T* slots, size_t slot_elems, int grid, cudaStream_t s);
+                                       T* slots, size_t slot_elems, int grid, int C, cudaStream_t s);
 
 }  // namespace jac

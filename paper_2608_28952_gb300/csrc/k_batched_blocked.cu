@@ -21,10 +21,15 @@
 // zero padding that is never rotated) live in a per-CTA slot of global
 // memory; the blocks a warp works on are staged through shared memory.
 #include <cuda_runtime.h>
+#include <algorithm>
 
 #include "batched.h"
 #include "cluster_common.cuh"
 #include "jacobi_core.cuh"
+
+#include <cooperative_groups.h>
+
+namespace cg = cooperative_groups;
 
 namespace jac {
 
@@ -166,21 +171,32 @@ __device__ int warp_pivot(BlkWarp<T>& w, T* V, T tol, int lane)
 template <typename T>
 __global__ void __launch_bounds__(blk_threads<T>()) k_batched_evd_blocked(BatchedEvdArgs<T> a, const int* list,
                                                                         int count, unsigned* queue, T* slots,
-                                                                        size_t slot_elems)
+                                                                        size_t slot_elems, int C)
 {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int cr = C > 1 ? (int)cluster.block_rank() : 0;
+    auto sync_all = [&] {
+        if (C > 1) cluster.sync();
+        else __syncthreads();
+    };
     extern __shared__ __align__(16) unsigned char bsm[];
     constexpr int VLD = sld<T>();
     T* Vs = (T*)bsm;                                          // [BMAXP][BK * VLD] pivot V's of the step
     BlkWarp<T>* warps = (BlkWarp<T>*)(Vs + (size_t)BMAXP * BK * VLD);
-    __shared__ int s_item, s_rot, s_prot[BMAXP];
+    __shared__ int s_item, s_rot, s_bad, s_prot[BMAXP];
     __shared__ unsigned long long s_flops;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    // thread and warp numbers over the CTAs that share the matrix
+    const int ctid = cr * blockDim.x + tid, cnt = C * blockDim.x, cwid = wid * C + cr, cnw = C * nw;
     BlkWarp<T>& w = warps[wid];
-    T* Aw = slots + (size_t)blockIdx.x * slot_elems;
+    T* Aw = slots + (size_t)(blockIdx.x / C) * slot_elems;
 
     for (;;) {
-        if (tid == 0) s_item = (int)atomicAdd(queue, 1u);
-        __syncthreads();
+        if (tid == 0 && cr == 0) {
+            const int it = (int)atomicAdd(queue, 1u);
+            for (int u = 0; u < C; ++u) *(C > 1 ? cluster.map_shared_rank(&s_item, u) : &s_item) = it;
+        }
+        sync_all();
         const int item = s_item;
         if (item >= count) break;
         const int mat = list[item];
@@ -192,7 +208,7 @@ __global__ void __launch_bounds__(blk_threads<T>()) k_batched_evd_blocked(Batche
         const size_t lda = (size_t)a.lda[mat];
         // ---- load: mirrored lower triangle, zero padding; Q = I
         int bad = 0;
-        for (size_t idx = tid; idx < (size_t)np * np; idx += blockDim.x) {
+        for (size_t idx = ctid; idx < (size_t)np * np; idx += cnt) {
             const int i = (int)(idx % np), j = (int)(idx / np);
             T v = T(0);
             if (i < n && j < n) {
@@ -205,14 +221,22 @@ __global__ void __launch_bounds__(blk_threads<T>()) k_batched_evd_blocked(Batche
         if (tid == 0) {
             s_rot = 0;
             s_flops = 0;
+            s_bad = 0;
         }
         bad = __syncthreads_or(bad);
+        if (C > 1) {
+            cluster.sync();
+            if (bad && tid == 0)
+                for (int u = 0; u < C; ++u) *cluster.map_shared_rank(&s_bad, u) = 1;
+            cluster.sync();
+            bad = s_bad;
+        }
         int sweeps = 0, last = 1;
         const int max_sweeps = bad ? 0 : a.max_sweeps;
         for (int sw = 0; sw < max_sweeps; ++sw) {
             for (int s = 0; s < N - 1; ++s) {
                 // ---- 1. pivot solves, one warp per pair
-                for (int e = wid; e < npairs; e += nw) {
+                for (int e = cwid; e < npairs; e += cnw) {
                     int I, J;
                     rr_pair(N, s, e, I, J);
                     T* V = Vs + (size_t)e * BK * VLD;   // accumulated column-major, ld BLD
@@ -265,21 +289,28 @@ __global__ void __launch_bounds__(blk_threads<T>()) k_batched_evd_blocked(Batche
                             for (int c = 0; c < BK; ++c) V[lane + BLD * w.dest[c]] = col[c];
                         }
                     }
+                    __syncwarp();
+                    if (rot > 0)   // V to the other CTAs of the matrix
+                        for (int u = 0; u < C; ++u) {
+                            if (u == cr) continue;
+                            T* Vr = cluster.map_shared_rank(V, u);
+                            for (int c = lane; c < BK * VLD; c += 32) Vr[c] = V[c];
+                        }
                     if (lane == 0) {
-                        s_prot[e] = rot;
+                        for (int u = 0; u < C; ++u) *(C > 1 ? cluster.map_shared_rank(&s_prot[e], u) : &s_prot[e]) = rot;
                         if (rot) {
-                            atomicAdd(&s_rot, rot);
                             // per applied rotation: its quads in the pivot (both sides) and a V column pair
                             atomicAdd(&s_flops, (unsigned long long)rot * 12ull * BK);
                         }
                     }
                     __syncwarp();
                 }
-                __syncthreads();
+                sync_all();
+                if (tid < npairs && s_prot[tid]) s_rot = 1;
                 // ---- 2. updates, one warp per item
                 const int npb = npairs * (npairs - 1) / 2;
                 const int nq = vec ? npairs * (np / BK) : 0;
-                for (int it = wid; it < npb + nq; it += nw) {
+                for (int it = cwid; it < npb + nq; it += cnw) {
                     T* S = w.tile;
                     if (it < npb) {
                         int e1, e2;
@@ -398,7 +429,7 @@ __global__ void __launch_bounds__(blk_threads<T>()) k_batched_evd_blocked(Batche
                         __syncwarp();
                     }
                 }
-                __syncthreads();
+                sync_all();
             }
             sweeps = sw + 1;
             last = s_rot;
@@ -417,27 +448,29 @@ __global__ void __launch_bounds__(blk_threads<T>()) k_batched_evd_blocked(Batche
                 const T dy = Aw[y + (size_t)np * y];
                 r += (dy < dx) || (dy == dx && y < x);
             }
-            wout[r] = dx;
+            if (cr == 0) wout[r] = dx;
             rank[x] = r;
         }
         __syncthreads();
         if (vec) {
             T* Q = a.Q[mat];
             const size_t ldq = (size_t)a.ldq[mat];
-            for (size_t idx = tid; idx < (size_t)n * n; idx += blockDim.x) {
+            for (size_t idx = ctid; idx < (size_t)n * n; idx += cnt) {
                 const int i = (int)(idx % n), j = (int)(idx / n);
                 Q[i + ldq * rank[j]] = Qw[i + (size_t)np * j];
             }
         }
         if (tid == 0) {
             const bool converged = !bad && last == 0;
-            a.info[mat] = bad ? -100 : (converged ? 0 : sweeps);
-            atomicAdd(&a.cnt->inner_sweeps, (unsigned long long)sweeps);
-            atomicAdd(&a.cnt->pair_solves, 1ull);
+            if (cr == 0) {
+                a.info[mat] = bad ? -100 : (converged ? 0 : sweeps);
+                atomicAdd(&a.cnt->inner_sweeps, (unsigned long long)sweeps);
+                atomicAdd(&a.cnt->pair_solves, 1ull);
+            }
             if (sizeof(T) == 8) atomicAdd(&a.cnt->flops_fp64, s_flops);
             else atomicAdd(&a.cnt->flops_fp32, s_flops);
         }
-        __syncthreads();
+        sync_all();
     }
 }
 
@@ -474,15 +507,26 @@ size_t batched_blocked_slot_elems(int nmax)
 
 template <typename T>
 cudaError_t launch_batched_evd_blocked(const BatchedEvdArgs<T>& a, const int* list, int count, unsigned* queue,
-                                       T* slots, size_t slot_elems, int grid, cudaStream_t s)
+                                       T* slots, size_t slot_elems, int grid, int C, cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
     const size_t smem = batched_blocked_smem<T>();
     cudaError_t e = cudaFuncSetAttribute(k_batched_evd_blocked<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(queue, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-    k_batched_evd_blocked<T><<<grid, blk_threads<T>(), smem, s>>>(a, list, count, queue, slots, slot_elems);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(grid / C, count) * C);
+    cfg.blockDim = dim3(blk_threads<T>());
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_batched_evd_blocked<T>, a, list, count, queue, slots, slot_elems, C);
 }
 
 template size_t batched_blocked_smem<float>();
@@ -492,8 +536,8 @@ template int batched_blocked_ctas_per_sm<double>();
 template size_t batched_blocked_slot_elems<float>(int);
 template size_t batched_blocked_slot_elems<double>(int);
 template cudaError_t launch_batched_evd_blocked<float>(const BatchedEvdArgs<float>&, const int*, int, unsigned*, float*,
-                                                       size_t, int, cudaStream_t);
+                                                       size_t, int, int, cudaStream_t);
 template cudaError_t launch_batched_evd_blocked<double>(const BatchedEvdArgs<double>&, const int*, int, unsigned*,
-                                                        double*, size_t, int, cudaStream_t);
+                                                        double*, size_t, int, int, cudaStream_t);
 
 }  // namespace jac
