@@ -14,8 +14,11 @@
  *   - matrices are column-major with a leading dimension (lda, ldq, ...);
  *   - pointers are DEVICE pointers unless the entry point name ends in "_h"
  *     (host pointers) or the argument is named h_*;
- *   - the caller owns every buffer; the library allocates its workspace with
- *     cudaMallocAsync on the given stream and frees it before returning;
+ *   - the caller owns every buffer; the library allocates its workspace
+ *     stream-ordered on the given stream and frees it before returning, from
+ *     a memory pool of its own per device that holds on to at most 8 GiB
+ *     between calls (the driver takes it back when an allocation of the
+ *     process would otherwise fail);
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *     stream); the calls return only after the work is complete;
  *   - nothing is printed, nothing throws, nothing exits;

@@ -39,7 +39,7 @@ struct Workspace {
             return nullptr;
         }
         void* p = nullptr;
-        if (cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
+        if (workspace_alloc(&p, bytes, s) != cudaSuccess) {
             failed = true;
             cudaGetLastError();
             return nullptr;

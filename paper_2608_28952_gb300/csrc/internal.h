@@ -273,4 +273,7 @@ cudaError_t launch_oa_step_elementwise(int np, const double* S, double* G, doubl
 cudaError_t launch_symmetrize(int np, const double* S, double* B, cudaStream_t s);
 cudaError_t launch_ns_halfres(int np, double* G, cudaStream_t s);
 
+// Stream-ordered allocation from the library's own pool (pool.cpp), freed with cudaFreeAsync.
+cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t s);
+
 }  // namespace jac

@@ -1195,7 +1195,7 @@ extern "C" int jacobi_f64emu_gemm(int M, int N, int K, const double* A, int lda,
     }
     int* err = nullptr;
     const bool big = K > 256;
-    if (cudaMallocAsync(&err, sizeof(int) * (1 + (big ? M + N : 0)), s) != cudaSuccess) return JACOBI_ERR_ALLOC;
+    if (jac::workspace_alloc((void**)&err, sizeof(int) * (1 + (big ? M + N : 0)), s) != cudaSuccess) return JACOBI_ERR_ALLOC;
     int h = 0, rc = 0;
     if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess ||
         (big ? jac::launch_emu_gemm_big(M, N, K, A, lda, transA, B, ldb, 0, C, ldc, 0, err + 1, err + 1 + M, err, s)

@@ -215,7 +215,7 @@ extern "C" int jacobi_lowp_gemm(int M, int N, int K, const float* A, int lda, in
         return 0;
     }
     int* err = nullptr;
-    if (cudaMallocAsync(&err, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_ALLOC;
+    if (jac::workspace_alloc((void**)&err, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_ALLOC;
     int h = 0;
     int rc = 0;
     if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess ||
