@@ -312,7 +312,9 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
     if (!make_ordering(p.ordering, N, &ord)) return -7;
     const bool vec = p.want_vectors != 0;
     const double tol = std::max(p.tol, sqrt((double)m) * U64);
-    const int npanels = gram_panels_for(m);
+    const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
+    const int prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, ord.dev_per_step, k);
+    const int npanels = (m + prows - 1) / prows;
     int rc = 0;
     {
         Workspace ws(s);
@@ -332,7 +334,6 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         DevCounters* cnt = ws.get<DevCounters>(1);
         const int pcl = choose_pivot_cluster(k, ord.dev_per_step);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
-        const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
         int* err = emu ? ws.get<int>(1) : nullptr;
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),
@@ -363,9 +364,9 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                 for (int si = 0; si < ord.S; ++si) {
                     const int nps = ord.dev_per_step, p0 = si * nps;
                     EmuSvdArgs sa{Gw[c], Gw[c ^ 1], m, m, Vw[c], Vw[c ^ 1], np, np, dpairs + p0, nps, b, k,
-                                  Vb, rot, part, npanels, gram_panel_rows(), err, cnt};
+                                  Vb, rot, part, npanels, prows, err, cnt};
                     if ((emu ? launch_emu_gram(sa, cs)
-                             : launch_gram(Gw[c], m, m, dpairs + p0, nps, b, k, part, cnt, cs)) != cudaSuccess)
+                             : launch_gram(Gw[c], m, m, dpairs + p0, nps, b, k, npanels, prows, part, cnt, cs)) != cudaSuccess)
                         return false;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 1], cs, cudaEventRecordExternal) != cudaSuccess) return false;
                     PivotArgs pa{};
@@ -797,8 +798,10 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
     if (!make_ordering(p.ordering, np / b, &ord)) return -2;
     if (step < 0 || step >= ord.S) return -8;
     const double tol = std::max(p.tol, sqrt((double)m) * U64);
-    const int npanels = gram_panels_for(m);
     const int nps = ord.dev_per_step, p0 = step * nps;
+    const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
+    const int prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, nps, k);
+    const int npanels = (m + prows - 1) / prows;
     {
         Workspace ws(s);
         double* Gw[2] = {ws.get<double>((size_t)m * np), ws.get<double>((size_t)m * np)};
@@ -815,7 +818,6 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         DevCounters* cnt = ws.get<DevCounters>(1);
         const int pcl = choose_pivot_cluster(k, nps);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
-        const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
         int* err = emu ? ws.get<int>(1) : nullptr;
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (err && cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
@@ -830,8 +832,8 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
                                    cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
         EmuSvdArgs sa{Gw[0], Gw[1], m, m, Vw[0], Vw[1], np, np, dpairs + p0, nps, b, k,
-                      Vb, rot, part, npanels, gram_panel_rows(), err, cnt};
-        if ((emu ? launch_emu_gram(sa, s) : launch_gram(Gw[0], m, m, dpairs + p0, nps, b, k, part, cnt, s)) !=
+                      Vb, rot, part, npanels, prows, err, cnt};
+        if ((emu ? launch_emu_gram(sa, s) : launch_gram(Gw[0], m, m, dpairs + p0, nps, b, k, npanels, prows, part, cnt, s)) !=
             cudaSuccess)
             return JACOBI_ERR_CUDA;
         PivotArgs pa{};

@@ -175,18 +175,35 @@ __global__ void __launch_bounds__(RED_T) k_offnorm(int np, const TA* __restrict_
         last = (t == (unsigned int)G - 1);
     }
     __syncthreads();
-    if (last && tid == 0) {
+    // the last CTA sums the partials in a fixed order: each thread a strided
+    // few, then the tree again (one thread adding up to 608 of them in turn
+    // was 64 cycles an addition: 45 of this kernel's 53 us at n = 256)
+    if (last) {
         __threadfence();
-        double o = 0.0, a = 0.0, r = 0.0;
-        for (int g = 0; g < G; ++g) {  // fixed order
-            o += ((volatile double*)partial)[3 * g + 0];
-            a += ((volatile double*)partial)[3 * g + 1];
-            r = fmax(r, ((volatile double*)partial)[3 * g + 2]);
+        off = all = rel = 0.0;
+        for (int g = tid; g < G; g += RED_T) {
+            off += ((volatile double*)partial)[3 * g + 0];
+            all += ((volatile double*)partial)[3 * g + 1];
+            rel = fmax(rel, ((volatile double*)partial)[3 * g + 2]);
         }
-        result[0] = o;
-        result[1] = a;
-        result[2] = sqrt(r);
-        *ticket = 0u;
+        s_off[tid] = off;
+        s_all[tid] = all;
+        s_rel[tid] = rel;
+        __syncthreads();
+        for (int w = RED_T / 2; w > 0; w >>= 1) {
+            if (tid < w) {
+                s_off[tid] += s_off[tid + w];
+                s_all[tid] += s_all[tid + w];
+                s_rel[tid] = fmax(s_rel[tid], s_rel[tid + w]);
+            }
+            __syncthreads();
+        }
+        if (tid == 0) {
+            result[0] = s_off[0];
+            result[1] = s_all[0];
+            result[2] = sqrt(s_rel[0]);
+            *ticket = 0u;
+        }
     }
 }
 
@@ -398,34 +415,46 @@ cudaError_t launch_pivot(const PivotArgs& a, int C, cudaStream_t s)
 }
 
 // ======================================================================== GEMM tiles
-// C(M x 32) += Aop(M x K) Bop(K x 32) on 256 threads: thread (ty = tid % 32,
-// tx = tid / 32) owns rows ty + 32 i (i < MR) and columns tx + 8 j (j < 4).
-// K is streamed through shared memory in chunks of KC.
-constexpr int UPD_T = 256, KC = 16, TN = 32, T_LD = TN + 1;
-
+// C(M x TN) += Aop(M x K) Bop(K x TN), TN = 8 NJ, on 256 threads: thread (ty =
+// tid % 32, tx = tid / 32) owns rows ty + 32 i (i < MR) and columns tx + 8 j
+// (j < NJ).  K is streamed through shared memory in chunks of KC<MR>.  Every
+// output is one chain of FMAs over k in order, whatever the tile.
+//
+// Tile width of the updates: 8 columns.  FP64 is so slow here (64 cycles an
+// instruction and warp) that the loads a narrow tile repeats cost nothing, while
+// narrow items fill the GPU in small steps, pad less when 2b is no multiple of
+// 32 and leave a shorter last wave.  Measured per step, 8 / 16 / 32 columns: n =
+// 64, b = 16: 12.1 / 16.7 / 24.9 us; n = 256, b = 16: 15.7 / 21.1 / 25.3; n = 300,
+// b = 20: 33 / 40 / 52; n = 500, b = 32: 65 / 74 / 107; n = 1024, b = 128: 805 /
+// 802 / 1555; n = 2048, b = 64: 1725 / 1740 / 1814; n = 4096, b = 64: 6.88 / 6.84 /
+// 6.92 ms.  (One width for all: the wider ones win nowhere by more than 0.5 %.)
+constexpr int UPD_T = 256, UPD_SMS = 152, UPD_NJ = 1;
 template <int MR>
+constexpr int KC = MR <= 2 ? 32 : 16;
+
+template <int MR, int NJ>
 struct Tile {
-    double acc[MR][4];
+    double acc[MR][NJ];
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
         for (int i = 0; i < MR; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+            for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0;
     }
 };
 
-// As: [KC][AS_LD], Bs: [KC][T_LD] (or B directly from a shared buffer).
+// As: [KC][32 MR + 1], Bs: [KC][TN + 1] (or B directly from a shared buffer).
 // fa(m, kk) loads Aop(m, kk); fb(kk, j) loads Bop(kk, j).  a_kfast / b_kfast
 // choose which index runs fastest across threads while loading (coalescing).
-template <int MR, bool A_KFAST, bool B_SMEM, bool B_KFAST, class FA, class FB>
-__device__ __forceinline__ void gemm_tile(Tile<MR>& t, int M, int K, int mr, FA fa, FB fb,
+template <int MR, int NJ, bool A_KFAST, bool B_SMEM, bool B_KFAST, class FA, class FB>
+__device__ __forceinline__ void gemm_tile(Tile<MR, NJ>& t, int M, int K, int mr, FA fa, FB fb,
                                           double* As, double* Bs, const double* Bsm)
 {
-    constexpr int AS_LD = 32 * MR + 1;
+    constexpr int AS_LD = 32 * MR + 1, TN = 8 * NJ, T_LD = TN + 1, KCT = KC<MR>;
     const int tid = threadIdx.x, ty = tid & 31, tx = tid >> 5;
-    for (int k0 = 0; k0 < K; k0 += KC) {
-        const int kc = min(KC, K - k0);
+    for (int k0 = 0; k0 < K; k0 += KCT) {
+        const int kc = min(KCT, K - k0);
         if (A_KFAST) {
             for (int idx = tid; idx < kc * M; idx += UPD_T) {
                 const int m = idx / kc, kk = idx - m * kc;
@@ -445,7 +474,7 @@ __device__ __forceinline__ void gemm_tile(Tile<MR>& t, int M, int K, int mr, FA 
                 }
             } else {
                 for (int idx = tid; idx < kc * TN; idx += UPD_T) {
-                    const int kk = idx >> 5, j = idx & 31;
+                    const int kk = idx / TN, j = idx - kk * TN;
                     Bs[kk * T_LD + j] = fb(k0 + kk, j);
                 }
             }
@@ -453,15 +482,15 @@ __device__ __forceinline__ void gemm_tile(Tile<MR>& t, int M, int K, int mr, FA 
         __syncthreads();
         const double* Bk = B_SMEM ? (Bsm + (size_t)k0 * T_LD) : Bs;
         for (int kk = 0; kk < kc; ++kk) {
-            double bv[4];
+            double bv[NJ];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Bk[kk * T_LD + tx + 8 * j];
+            for (int j = 0; j < NJ; ++j) bv[j] = Bk[kk * T_LD + tx + 8 * j];
 #pragma unroll
             for (int i = 0; i < MR; ++i) {
                 if (i < mr) {
                     const double av = As[kk * AS_LD + ty + 32 * i];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) t.acc[i][j] = fma(av, bv[j], t.acc[i][j]);
+                    for (int j = 0; j < NJ; ++j) t.acc[i][j] = fma(av, bv[j], t.acc[i][j]);
                 }
             }
         }
@@ -469,11 +498,11 @@ __device__ __forceinline__ void gemm_tile(Tile<MR>& t, int M, int K, int mr, FA 
     }
 }
 
-template <int MR>
-static size_t update_smem_bytes()
+// shared memory of one item: the A and B chunks, and (update_evd) T
+template <int MR, int NJ>
+static size_t tile_smem_bytes(bool with_t)
 {
-    return ((size_t)KC * (32 * MR + 1) + (size_t)KC * T_LD + (size_t)(32 * MR) * T_LD) *
-           sizeof(double);
+    return ((size_t)KC<MR> * (32 * MR + 1 + 8 * NJ + 1) + (with_t ? (size_t)(32 * MR) * (8 * NJ + 1) : 0)) * sizeof(double);
 }
 
 // ======================================================================== EVD update
@@ -486,18 +515,18 @@ __device__ __forceinline__ void decode_pairblock(int pb, int& e1, int& e2)
     e1 = pb - t * (t - 1) / 2;
 }
 
-template <int MR>
+template <int MR, int NJ>
 __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_sand, int nchunks)
 {
     extern __shared__ __align__(16) double sm[];
-    constexpr int AS_LD = 32 * MR + 1;
+    constexpr int AS_LD = 32 * MR + 1, TN = 8 * NJ, T_LD = TN + 1;
     double* As = sm;
-    double* Bs = As + KC * AS_LD;
-    double* Ts = Bs + KC * T_LD;  // [32*MR][T_LD]
+    double* Bs = As + KC<MR> * AS_LD;
+    double* Ts = Bs + KC<MR> * T_LD;  // [32*MR][T_LD]
     const int tid = threadIdx.x, ty = tid & 31, tx = tid >> 5;
     const int k = a.k, b = a.b;
     const int item = blockIdx.x;
-    Tile<MR> t;
+    Tile<MR, NJ> t;
 
     if (item < n_sand) {
         // ---------------- A'_{P1P2} (:, chunk) = V1^T (A_{P1P2} V2(:, chunk))
@@ -517,7 +546,7 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_san
         // stage 1: T = A_blk V2(:, chunk)  (or the plain chunk when V2 == I)
         if (r2) {
             t.zero();
-            gemm_tile<MR, false, false, true>(
+            gemm_tile<MR, NJ, false, false, true>(
                 t, k, k, mr,
                 [&](int m, int kk) { return Ain[pair_map(I1, J1, b, m) + (size_t)lda * pair_map(I2, J2, b, kk)]; },
                 [&](int kk, int j) { return j < kw ? V2[kk + (size_t)k * (c0 + j)] : 0.0; }, As, Bs,
@@ -525,7 +554,7 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_san
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+                for (int j = 0; j < NJ; ++j)
                     if (i < mr) Ts[(ty + 32 * i) * T_LD + tx + 8 * j] = t.acc[i][j];
         } else {
             for (int idx = tid; idx < k * TN; idx += UPD_T) {
@@ -537,13 +566,13 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_san
         // stage 2: O = V1^T T
         if (r1) {
             t.zero();
-            gemm_tile<MR, false, true, false>(
+            gemm_tile<MR, NJ, false, true, false>(
                 t, k, k, mr, [&](int m, int kk) { return V1t[m + (size_t)k * kk]; },
                 [&](int, int) { return 0.0; }, As, Bs, Ts);
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < NJ; ++j) {
                     const int m = ty + 32 * i, jj = tx + 8 * j;
                     if (i < mr && m < k && jj < kw) {
                         const int gi = pair_map(I1, J1, b, m), gj = pair_map(I2, J2, b, c0 + jj);
@@ -586,14 +615,14 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_san
         const double* Vp = a.V + (size_t)e * 2 * k * k;
         if (r) {
             t.zero();
-            gemm_tile<MR, false, false, true>(
+            gemm_tile<MR, NJ, false, false, true>(
                 t, M, k, mr, [&](int m, int kk) { return Qin[(r0 + m) + (size_t)ldq * pair_map(I, J, b, kk)]; },
                 [&](int kk, int j) { return j < kw ? Vp[kk + (size_t)k * (c0 + j)] : 0.0; }, As, Bs,
                 nullptr);
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < NJ; ++j) {
                     const int m = ty + 32 * i, jj = tx + 8 * j;
                     if (i < mr && m < M && jj < kw)
                         a.Qout[(r0 + m) + (size_t)ldq * pair_map(I, J, b, c0 + jj)] = t.acc[i][j];
@@ -612,38 +641,38 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_san
     }
 }
 
-template <int MR>
-static cudaError_t launch_update_evd_mr(const UpdateArgs& a, cudaStream_t s)
+template <int MR, int NJ>
+static cudaError_t launch_update_evd_t(const UpdateArgs& a, cudaStream_t s)
 {
-    const int nchunks = (a.k + TN - 1) / TN;
+    const int nchunks = (a.k + 8 * NJ - 1) / (8 * NJ);
     const int n_sand = a.npairs * (a.npairs - 1) / 2 * nchunks;
     const int H = 32 * MR;
     const int n_q = a.Qin ? a.npairs * ((a.qrows + H - 1) / H) * nchunks : 0;
     const int items = n_sand + n_q;
     if (items == 0) return cudaSuccess;
-    const size_t smem = update_smem_bytes<MR>();
-    cudaError_t e = cudaFuncSetAttribute(k_update_evd<MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = tile_smem_bytes<MR, NJ>(true);
+    cudaError_t e = cudaFuncSetAttribute(k_update_evd<MR, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_update_evd<MR><<<items, UPD_T, smem, s>>>(a, n_sand, nchunks);
+    k_update_evd<MR, NJ><<<items, UPD_T, smem, s>>>(a, n_sand, nchunks);
     return cudaGetLastError();
 }
 
 cudaError_t launch_update_evd(const UpdateArgs& a, cudaStream_t s)
 {
-    if (a.k <= 32) return launch_update_evd_mr<1>(a, s);
-    if (a.k <= 64) return launch_update_evd_mr<2>(a, s);
-    if (a.k <= 128) return launch_update_evd_mr<4>(a, s);
-    return launch_update_evd_mr<8>(a, s);
+    if (a.k <= 32) return launch_update_evd_t<1, UPD_NJ>(a, s);
+    if (a.k <= 64) return launch_update_evd_t<2, UPD_NJ>(a, s);
+    if (a.k <= 128) return launch_update_evd_t<4, UPD_NJ>(a, s);
+    return launch_update_evd_t<8, UPD_NJ>(a, s);
 }
 
 // ======================================================================== one-sided column update
-template <int MR>
+template <int MR, int NJ>
 __global__ void __launch_bounds__(UPD_T, 2) k_update_cols(ColUpdateArgs a, int n_g, int nchunks)
 {
     extern __shared__ __align__(16) double sm[];
-    constexpr int AS_LD = 32 * MR + 1;
+    constexpr int AS_LD = 32 * MR + 1, TN = 8 * NJ, T_LD = TN + 1;
     double* As = sm;
-    double* Bs = As + KC * AS_LD;
+    double* Bs = As + KC<MR> * AS_LD;
     const int tid = threadIdx.x, ty = tid & 31, tx = tid >> 5;
     const int k = a.k, b = a.b, H = 32 * MR;
     int item = blockIdx.x;
@@ -667,15 +696,15 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_cols(ColUpdateArgs a, int n
     const int mr = (M + 31) >> 5;
     const double* Vp = a.Vh + (size_t)e * 2 * k * k;
     if (r) {
-        Tile<MR> t;
+        Tile<MR, NJ> t;
         t.zero();
-        gemm_tile<MR, false, false, true>(
+        gemm_tile<MR, NJ, false, false, true>(
             t, M, k, mr, [&](int m, int kk) { return Min[(r0 + m) + (size_t)ld * pair_map(I, J, b, kk)]; },
             [&](int kk, int j) { return j < kw ? Vp[kk + (size_t)k * (c0 + j)] : 0.0; }, As, Bs, nullptr);
 #pragma unroll
         for (int i = 0; i < MR; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < NJ; ++j) {
                 const int m = ty + 32 * i, jj = tx + 8 * j;
                 if (i < mr && m < M && jj < kw)
                     Mout[(r0 + m) + (size_t)ld * pair_map(I, J, b, c0 + jj)] = t.acc[i][j];
@@ -693,43 +722,53 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_cols(ColUpdateArgs a, int n
     }
 }
 
-template <int MR>
-static cudaError_t launch_update_cols_mr(const ColUpdateArgs& a, cudaStream_t s)
+template <int MR, int NJ>
+static cudaError_t launch_update_cols_t(const ColUpdateArgs& a, cudaStream_t s)
 {
-    const int nchunks = (a.k + TN - 1) / TN, H = 32 * MR;
+    const int nchunks = (a.k + 8 * NJ - 1) / (8 * NJ), H = 32 * MR;
     const int n_g = a.npairs * ((a.m + H - 1) / H) * nchunks;
     const int n_v = a.Vin ? a.npairs * ((a.vrows + H - 1) / H) * nchunks : 0;
     if (n_g + n_v == 0) return cudaSuccess;
-    const size_t smem = ((size_t)KC * (32 * MR + 1) + (size_t)KC * T_LD) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_update_cols<MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = tile_smem_bytes<MR, NJ>(false);
+    cudaError_t e = cudaFuncSetAttribute(k_update_cols<MR, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_update_cols<MR><<<n_g + n_v, UPD_T, smem, s>>>(a, n_g, nchunks);
+    k_update_cols<MR, NJ><<<n_g + n_v, UPD_T, smem, s>>>(a, n_g, nchunks);
     return cudaGetLastError();
 }
 
+// Tiles of 128 rows (fewer loads of Vhat) while they fill the GPU, else of 32.
 cudaError_t launch_update_cols(const ColUpdateArgs& a, cudaStream_t s)
 {
-    // tiles of 128 rows: the inner dimension is k, so a 128 x 32 tile costs 2*128*32*k
-    return launch_update_cols_mr<4>(a, s);
+    const int tiles = a.npairs * ((a.m + 127) / 128 + (a.Vin ? (a.vrows + 127) / 128 : 0)) * ((a.k + 7) / 8);
+    return tiles >= 8 * UPD_SMS ? launch_update_cols_t<4, UPD_NJ>(a, s) : launch_update_cols_t<1, UPD_NJ>(a, s);
 }
 
 // ======================================================================== Gram (split K over rows)
 constexpr int GRAM_ROWS = 512;
 int gram_panel_rows() { return GRAM_ROWS; }
-int gram_panels_for(int m) { return (m + GRAM_ROWS - 1) / GRAM_ROWS; }
+// Rows of a panel for the FP64 Gram blocks: 512 (few partials to sum) while the
+// panels fill the GPU, else as few as 64 (a 512-row panel of a 32 x 32 block is
+// 126 us of one SM; 7 pairs of 1000 rows were 14 such items: 1000 x 200, b = 16,
+// Gram and update 202 -> 41 us per step).
+int gram_panel_rows_for(int m, int npairs, int k)
+{
+    int rows = GRAM_ROWS;
+    while (rows > 64 && npairs * ((m + rows - 1) / rows) * ((k + 31) / 32) < 2 * UPD_SMS) rows /= 2;
+    return rows;
+}
 
 // Item (pair e, panel r, column chunk c): rows c0.. of the k x k Gram block
 // (lower triangle only: rows >= c0), K = the panel's rows of G.
-template <int MR>
+template <int MR, int NJ>
 __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G, int ldg, int m,
                                                   const int2* __restrict__ pairs, int b, int k,
-                                                  int npanels, int nchunks, double* __restrict__ part,
+                                                  int npanels, int prows, int nchunks, double* __restrict__ part,
                                                   DevCounters* cnt)
 {
     extern __shared__ __align__(16) double sm[];
-    constexpr int AS_LD = 32 * MR + 1;
+    constexpr int AS_LD = 32 * MR + 1, TN = 8 * NJ, T_LD = TN + 1;
     double* As = sm;
-    double* Bs = As + KC * AS_LD;
+    double* Bs = As + KC<MR> * AS_LD;
     const int tid = threadIdx.x, ty = tid & 31, tx = tid >> 5;
     const int item = blockIdx.x;
     const int c = item % nchunks;
@@ -740,10 +779,10 @@ __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G,
     const int c0 = c * TN, kw = min(TN, k - c0);
     const int row0 = c0;  // lower triangle: output rows >= first column of the chunk
     const int M = k - row0, mr = (M + 31) >> 5;
-    const int g0 = pr * GRAM_ROWS, K = min(GRAM_ROWS, m - g0);
-    Tile<MR> t;
+    const int g0 = pr * prows, K = min(prows, m - g0);
+    Tile<MR, NJ> t;
     t.zero();
-    gemm_tile<MR, true, false, true>(
+    gemm_tile<MR, NJ, true, false, true>(
         t, M, K, mr,
         [&](int mm, int kk) { return G[(g0 + kk) + (size_t)ldg * pair_map(I, J, b, row0 + mm)]; },
         [&](int kk, int j) { return j < kw ? G[(g0 + kk) + (size_t)ldg * pair_map(I, J, b, c0 + j)] : 0.0; },
@@ -752,7 +791,7 @@ __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G,
 #pragma unroll
     for (int i = 0; i < MR; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < NJ; ++j) {
             const int mm = ty + 32 * i, jj = tx + 8 * j;
             if (i < mr && mm < M && jj < kw) out[(row0 + mm) + (size_t)k * (c0 + jj)] = t.acc[i][j];
         }
@@ -762,25 +801,27 @@ __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G,
     }
 }
 
-cudaError_t launch_gram(const double* G, int ldg, int m, const int2* pairs, int npairs, int b,
-                        int k, double* part, DevCounters* cnt, cudaStream_t s)
+template <int MR, int NJ>
+static cudaError_t launch_gram_t(const double* G, int ldg, int m, const int2* pairs, int npairs, int b, int k, int npanels,
+                                 int prows, double* part, DevCounters* cnt, cudaStream_t s)
 {
-    const int nchunks = (k + TN - 1) / TN, npanels = gram_panels_for(m);
-    const int items = npairs * npanels * nchunks;
-    if (items == 0) return cudaSuccess;
-#define JAC_GRAM(MR)                                                                               \
-    do {                                                                                           \
-        const size_t smem = ((size_t)KC * (32 * MR + 1) + (size_t)KC * T_LD) * sizeof(double);     \
-        cudaError_t e = cudaFuncSetAttribute(k_gram<MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-        if (e != cudaSuccess) return e;                                                            \
-        k_gram<MR><<<items, UPD_T, smem, s>>>(G, ldg, m, pairs, b, k, npanels, nchunks, part, cnt); \
-    } while (0)
-    if (k <= 32) JAC_GRAM(1);
-    else if (k <= 64) JAC_GRAM(2);
-    else if (k <= 128) JAC_GRAM(4);
-    else JAC_GRAM(8);
-#undef JAC_GRAM
+    const int nchunks = (k + 8 * NJ - 1) / (8 * NJ);
+    const size_t smem = tile_smem_bytes<MR, NJ>(false);
+    cudaError_t e = cudaFuncSetAttribute(k_gram<MR, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_gram<MR, NJ><<<npairs * npanels * nchunks, UPD_T, smem, s>>>(G, ldg, m, pairs, b, k, npanels, prows, nchunks, part, cnt);
     return cudaGetLastError();
+}
+
+cudaError_t launch_gram(const double* G, int ldg, int m, const int2* pairs, int npairs, int b, int k, int npanels, int prows,
+                        double* part, DevCounters* cnt, cudaStream_t s)
+{
+    if (npairs * npanels == 0) return cudaSuccess;
+    auto go = [&](auto f) { return f(G, ldg, m, pairs, npairs, b, k, npanels, prows, part, cnt, s); };
+    if (k <= 32) return go(launch_gram_t<1, UPD_NJ>);
+    if (k <= 64) return go(launch_gram_t<2, UPD_NJ>);
+    if (k <= 128) return go(launch_gram_t<4, UPD_NJ>);
+    return go(launch_gram_t<8, UPD_NJ>);
 }
 
 // ======================================================================== general FP64 GEMM
@@ -795,16 +836,16 @@ __global__ void __launch_bounds__(UPD_T, 2) k_gemm64(int M, int N, int K, double
                                                      double* __restrict__ C, int ldc, int lower)
 {
     extern __shared__ __align__(16) double sm[];
-    constexpr int MR = 4, AS_LD = 32 * MR + 1;
+    constexpr int MR = 4, AS_LD = 32 * MR + 1, TN = 32;
     double* As = sm;
-    double* Bs = As + KC * AS_LD;
+    double* Bs = As + KC<MR> * AS_LD;
     const int tid = threadIdx.x, ty = tid & 31, tx = tid >> 5;
     const int m0 = blockIdx.x * 128, n0 = blockIdx.y * TN;
     if (lower && n0 >= m0 + 128) return;
     const int Mt = min(128, M - m0), mr = (Mt + 31) >> 5;
-    Tile<MR> t;
+    Tile<MR, 4> t;
     t.zero();
-    gemm_tile<MR, TRANS, false, true>(
+    gemm_tile<MR, 4, TRANS, false, true>(
         t, Mt, K, mr,
         [&](int m, int kk) { return TRANS ? A[kk + (size_t)lda * (m0 + m)] : A[(m0 + m) + (size_t)lda * kk]; },
         [&](int kk, int j) { return n0 + j < N ? B[kk + (size_t)ldb * (n0 + j)] : 0.0; }, As, Bs, nullptr);
@@ -850,8 +891,8 @@ cudaError_t launch_gemm64(int M, int N, int K, double alpha, const double* A, in
                           const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s,
                           int lower)
 {
-    const size_t smem = ((size_t)KC * (32 * 4 + 1) + (size_t)KC * T_LD) * sizeof(double);
-    dim3 grid((M + 127) / 128, (N + TN - 1) / TN);
+    const size_t smem = tile_smem_bytes<4, 4>(false);
+    dim3 grid((M + 127) / 128, (N + 31) / 32);
     cudaError_t e;
     if (transA) {
         if ((e = cudaFuncSetAttribute(k_gemm64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
@@ -864,28 +905,37 @@ cudaError_t launch_gemm64(int M, int N, int K, double alpha, const double* A, in
 }
 
 // ======================================================================== finalisation
-// Stable rank of key[i] among key[0..n): ascending (asc) or descending.
-__global__ void k_rank(int n, const double* __restrict__ key, int stride, int asc,
-                       int* __restrict__ rank)
+// Stable rank of key[i] among key[0..n): ascending (asc) or descending.  Keys
+// are compared as integers (an order-preserving map of the doubles, -0 and
+// +0 alike), 8 threads to a key: FP64 comparisons, one thread per key, took
+// 41 us at n = 256.
+__device__ __forceinline__ long long order_key(double x)
 {
-    __shared__ double tile[256];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const double ki = i < n ? key[(size_t)i * stride] : 0.0;
+    const long long v = __double_as_longlong(x + 0.0);
+    return v < 0 ? (long long)0x8000000000000000ull - v : v;
+}
+
+__global__ void __launch_bounds__(256) k_rank(int n, const double* __restrict__ key, int stride, int asc,
+                                              int* __restrict__ rank)
+{
+    __shared__ long long tile[256];
+    const int i = blockIdx.x * 32 + (threadIdx.x >> 3), part = threadIdx.x & 7;
+    const long long ki = i < n ? order_key(key[(size_t)i * stride]) : 0;
     int r = 0;
     for (int j0 = 0; j0 < n; j0 += 256) {
         const int j = j0 + threadIdx.x;
-        tile[threadIdx.x] = j < n ? key[(size_t)j * stride] : 0.0;
+        tile[threadIdx.x] = j < n ? order_key(key[(size_t)j * stride]) : 0;
         __syncthreads();
         const int lim = min(256, n - j0);
-        for (int u = 0; u < lim; ++u) {
-            const double kj = tile[u];
-            const int jj = j0 + u;
-            const bool before = asc ? (kj < ki || (kj == ki && jj < i)) : (kj > ki || (kj == ki && jj < i));
-            r += before;
+        for (int u = part; u < lim; u += 8) {
+            const long long kj = tile[u];
+            const bool before = asc ? kj < ki : kj > ki;
+            r += before || (kj == ki && j0 + u < i);
         }
         __syncthreads();
     }
-    if (i < n) rank[i] = r;
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (i < n && part == 0) rank[i] = r;
 }
 
 __global__ void k_finalize_evd(int n, int np, const double* __restrict__ Aw,
@@ -907,7 +957,7 @@ cudaError_t launch_finalize_evd(int n, int np, const double* Aw, const double* Q
                                 double* Q, int ldq, double* A, int lda, int* rank_ws,
                                 cudaStream_t s)
 {
-    k_rank<<<(n + 255) / 256, 256, 0, s>>>(n, Aw, np + 1, 1, rank_ws);
+    k_rank<<<(n + 31) / 32, 256, 0, s>>>(n, Aw, np + 1, 1, rank_ws);
     long long total = (long long)n * n;
     int blocks = (int)((total + 255) / 256);
     if (blocks > 152 * 16) blocks = 152 * 16;
@@ -960,7 +1010,7 @@ cudaError_t launch_finalize_svd(int m, int n, const double* Gw, int ldgw, const 
                                 double* norms_ws, int* rank_ws, cudaStream_t s)
 {
     k_colnorm<<<n, 256, 0, s>>>(m, Gw, ldgw, norms_ws);
-    k_rank<<<(n + 255) / 256, 256, 0, s>>>(n, norms_ws, 1, 0, rank_ws);
+    k_rank<<<(n + 31) / 32, 256, 0, s>>>(n, norms_ws, 1, 0, rank_ws);
     long long total = (long long)m * n + (V ? (long long)n * n : 0);
     int blocks = (int)((total + 255) / 256);
     if (blocks > 152 * 16) blocks = 152 * 16;
