@@ -24,66 +24,95 @@ namespace {
 constexpr int QR_T = 1024;   // threads of the column kernels
 constexpr int QR_KR = 512;   // rows per split of the Y^T X products
 
-__device__ double block_reduce(double v, double* red, bool is_max)
+// Sum over the CTA in a fixed order, the result in every thread.  A tree over
+// shared memory down to one warp: 32 dense warp additions where shuffles in
+// every warp would take 160 (an FP64 instruction holds the unit for 18 cycles
+// however few of its lanes count).
+__device__ double block_sum(double v, double* red)   // red: QR_T + 1 doubles
 {
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        const double u = __shfl_down_sync(0xffffffffu, v, o);
-        v = is_max ? fmax(v, u) : v + u;
+    const int tid = threadIdx.x;
+    red[tid] = v;
+    __syncthreads();
+#pragma unroll
+    for (int w = QR_T / 2; w >= 32; w >>= 1) {
+        if (tid < w) red[tid] += red[tid + w];
+        __syncthreads();
     }
+    if (tid < 32) {
+        v = red[tid];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (tid == 0) red[QR_T] = v;
+    }
+    __syncthreads();
+    return red[QR_T];
+}
+
+// The largest of nonnegative doubles, compared as integers.
+__device__ double block_max_abs(unsigned long long v, unsigned long long* red)   // red: 33 words
+{
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    for (int o = 16; o > 0; o >>= 1) v = max(v, (unsigned long long)__shfl_down_sync(0xffffffffu, v, o));
     if (lane == 0) red[w] = v;
     __syncthreads();
     if (w == 0) {
-        v = lane < nw ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            const double u = __shfl_down_sync(0xffffffffu, v, o);
-            v = is_max ? fmax(v, u) : v + u;
-        }
+        v = red[lane];
+        for (int o = 16; o > 0; o >>= 1) v = max(v, (unsigned long long)__shfl_down_sync(0xffffffffu, v, o));
         if (lane == 0) red[32] = v;
     }
     __syncthreads();
-    const double r = red[32];
-    __syncthreads();
-    return r;
+    return __longlong_as_double((long long)red[32]);
 }
+__device__ __forceinline__ unsigned long long abs_bits(double x) { return (unsigned long long)__double_as_longlong(x) & ~(1ull << 63); }
 
 // Householder vector of x = A(i:m, i): A(i, i) <- beta, Y(j0:m, i) <- v (zero
-// above row i), tau[i] <- tau.  One CTA.
+// above row i), tau[i] <- tau.  One CTA.  Its divisions and square roots are
+// one thread's work (all 1024 threads repeating them were 14 of 26 us at m =
+// 8192: the FP64 unit serves one warp instruction per 18 cycles).
 __global__ void __launch_bounds__(QR_T) k_house_vec(int m, double* __restrict__ A, int lda, int i,
                                                     double* __restrict__ Y, int ldy, int j0,
                                                     double* __restrict__ tau)
 {
-    __shared__ double red[33];
+    __shared__ double red[QR_T + 1];
+    __shared__ unsigned long long redm[33];
+    __shared__ double s_scale, s_sc;
     const int tid = threadIdx.x;
     const double* x = A + (size_t)lda * i;
-    const double alpha = x[i];
-    double mx = 0.0;
-    for (int r = i + 1 + tid; r < m; r += QR_T) mx = fmax(mx, fabs(x[r]));
-    mx = block_reduce(mx, red, true);
-    double xnorm = 0.0;
-    if (mx > 0.0) {   // ||tail|| = mx ||tail / mx||, no overflow or underflow in the squares
-        const double inv = 1.0 / mx;
-        double ss = 0.0;
+    unsigned long long top = 0;
+    for (int r = i + 1 + tid; r < m; r += QR_T) top = max(top, abs_bits(x[r]));
+    const double mx = block_max_abs(top, redm);
+    // ||tail||: the squares of x itself where none can overflow or vanish
+    // against the largest, else of x / mx
+    const bool plain = mx > 1e-140 && mx < 1e140;
+    if (!plain && mx > 0.0) {
+        if (tid == 0) s_scale = 1.0 / mx;
+        __syncthreads();
+    }
+    double ss = 0.0;
+    if (mx > 0.0) {
         for (int r = i + 1 + tid; r < m; r += QR_T) {
-            const double y = x[r] * inv;
+            const double y = plain ? x[r] : x[r] * s_scale;
             ss = fma(y, y, ss);
         }
-        xnorm = mx * sqrt(block_reduce(ss, red, false));
+        ss = block_sum(ss, red);
     }
     double* y = Y + (size_t)ldy * i;
-    if (xnorm == 0.0) {   // already reduced: H = I
-        if (tid == 0) tau[i] = 0.0;
-        for (int r = j0 + tid; r < m; r += QR_T) y[r] = r == i ? 1.0 : 0.0;
-        return;
-    }
-    const double big = fmax(fabs(alpha), xnorm), sml = fmin(fabs(alpha), xnorm), q = sml / big;
-    const double h = big * sqrt(fma(q, q, 1.0));
-    const double beta = alpha >= 0.0 ? -h : h;
-    const double sc = 1.0 / (alpha - beta);
     if (tid == 0) {
-        tau[i] = (beta - alpha) / beta;
-        A[i + (size_t)lda * i] = beta;
+        const double alpha = x[i];
+        const double xnorm = plain ? sqrt(ss) : (mx > 0.0 ? mx * sqrt(ss) : 0.0);
+        double sc = 0.0, t = 0.0;
+        if (xnorm != 0.0) {
+            const double big = fmax(fabs(alpha), xnorm), sml = fmin(fabs(alpha), xnorm), q = sml / big;
+            const double h = big * sqrt(fma(q, q, 1.0));
+            const double beta = alpha >= 0.0 ? -h : h;
+            sc = 1.0 / (alpha - beta);
+            t = (beta - alpha) / beta;
+            A[i + (size_t)lda * i] = beta;
+        }
+        tau[i] = t;   // 0: already reduced, H = I
+        s_sc = sc;
     }
+    __syncthreads();
+    const double sc = s_sc;
     for (int r = j0 + tid; r < m; r += QR_T) y[r] = r < i ? 0.0 : (r == i ? 1.0 : x[r] * sc);
 }
 
@@ -94,14 +123,14 @@ __global__ void __launch_bounds__(QR_T) k_house_apply(int m, double* __restrict_
                                                       int nrest, const double* __restrict__ Y, int ldy,
                                                       const double* __restrict__ tau, double* __restrict__ S)
 {
-    __shared__ double red[33];
+    __shared__ double red[QR_T + 1];
     const int tid = threadIdx.x, c = blockIdx.x, ii = i - j0;
     const double* v = Y + (size_t)ldy * i;
     if (c < nrest) {
         double* col = A + (size_t)lda * (i + 1 + c);
         double d = 0.0;
         for (int r = i + tid; r < m; r += QR_T) d = fma(v[r], col[r], d);
-        const double w = tau[i] * block_reduce(d, red, false);
+        const double w = tau[i] * block_sum(d, red);
         if (w != 0.0)
             for (int r = i + tid; r < m; r += QR_T) col[r] = fma(-w, v[r], col[r]);
     } else {
@@ -109,7 +138,7 @@ __global__ void __launch_bounds__(QR_T) k_house_apply(int m, double* __restrict_
         const double* yk = Y + (size_t)ldy * (j0 + kk);
         double d = 0.0;
         for (int r = i + tid; r < m; r += QR_T) d = fma(yk[r], v[r], d);
-        d = block_reduce(d, red, false);
+        d = block_sum(d, red);
         if (tid == 0) S[kk + QR_NB * ii] = d;
     }
 }
