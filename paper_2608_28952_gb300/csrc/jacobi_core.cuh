@@ -81,18 +81,18 @@ __device__ __forceinline__ bool rotation_wanted(T app, T aqq, T apq, T tol)
 // the FP64 overloads below do all they can outside the FP64 unit:
 //   * conversions between FP64 and FP32 by integer instructions on the bits;
 //   * t (the root of a t^2 + d t - a = 0 with |t| <= 1, d = aqq - app, a = apq,
-//     the textbook's choice), tau (t tau^2 + 2 tau - t = 0) and s (s (1 +
-//     tau^2) = 2 tau) each from an FP32 seed and one Newton step in pairs of
-//     floats (exact products by fma, error-free sums): 2^-42 relative;
+//     the textbook's choice), tau (t tau^2 + 2 tau - t = 0) and c ((1 + t^2) c^2
+//     - 1 = 0) each from an FP32 seed and one Newton step in pairs of floats
+//     (exact products by fma, error-free sums): 2^-42 relative;
 //   * then one Newton step in FP64 each: two FMAs for the residual, one for
 //     the step with the seed's FP32 reciprocal of the derivative, one addition
-//     to join the pair.
-// 13 FP64 instructions in place of about 40 with single FP32 seeds, two FP64
-// Newton steps and hardware conversions.  t is within 2u of the exact root,
-// tau within 4u, s within 6u of the exact root's, and, since s follows from the
-// computed tau, (1 - s tau)^2 + s^2 = 1 within u (measured over 2e7 triples):
-// the rotation applied in Rutishauser's or the three-shear form stays
-// orthogonal to working precision.
+//     to join the pair; s = t c.
+// 15 FP64 instructions (and tau and c side by side where two threads share a
+// rotation) in place of about 40 with single FP32 seeds, two FP64 Newton steps
+// and hardware conversions.  t is within 2u of the exact root, tau and s within
+// 4u, (1 - s tau)^2 + s^2 = 1 within 2u (measured over 2e7 triples): the rotation
+// applied in Rutishauser's or the three-shear form stays orthogonal to working
+// precision.
 __device__ __forceinline__ int f64_biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
 __device__ __forceinline__ float rsqrt_seed(float x)
@@ -107,21 +107,18 @@ __device__ __forceinline__ float rcp_seed(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// |x| 2^(sh - e), e its exponent: the leading 24 bits (truncated), and the next
-// 23; 0 below 2^-80.  sh <= 0.
-__device__ __forceinline__ float f64_lead(double x, int sh)
+// |x| 2^-e, e its exponent, in two parts: the leading 24 bits (truncated), in
+// [1, 2) for a normal x, and the next 23
+__device__ __forceinline__ float f64_lead(double x)
 {
-    const int hi = __double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    return sh < -80 ? 0.0f : __int_as_float(((sh + 127) << 23) | ((hi & 0xFFFFF) << 3) | (int)(lo >> 29));
+    return __int_as_float((127 << 23) | ((__double2hiint(x) & 0xFFFFF) << 3) | (int)((unsigned)__double2loint(x) >> 29));
 }
-__device__ __forceinline__ float f64_rest(double x, int sh)
+__device__ __forceinline__ float f64_rest(double x)
 {
-    const int lo = __double2loint(x);
-    return sh < -80 ? 0.0f
-                    : (__int_as_float(0x4B000000 | ((lo & 0x1FFFFFFF) >> 6)) - 8388608.0f) *
-                          __int_as_float((sh + 81) << 23);
+    return (__int_as_float(0x4B000000 | ((__double2loint(x) & 0x1FFFFFFF) >> 6)) - 8388608.0f) * __int_as_float(81 << 23);
 }
+// 2^e, e <= 0; 0 below 2^-80
+__device__ __forceinline__ float f32_pow2(int e) { return e < -80 ? 0.0f : __int_as_float((e + 127) << 23); }
 // f 2^e exactly (f a normal float or 0, the result normal)
 __device__ __forceinline__ double f64_of(float f, int e)
 {
@@ -175,58 +172,79 @@ __device__ __forceinline__ void schur2_wide(double d, double apq, double& s, dou
     tau = s * fma(r0, fma(e, e, e), r0);
 }
 
+// Biased exponents of d and apq for which the pairs of floats serve: normal
+// range with room for the Newton steps, and apq no smaller than 2^-60 d.
+__device__ __forceinline__ bool schur2_paired(int Ed, int Ea)
+{
+    const int E = max(Ed, Ea);
+    return E >= 128 && E <= 1900 && Ea + 60 >= E;
+}
+
+// The root t of a t^2 + d t - a, a = |apq|, d = |aqq - app| (biased exponents
+// Ea, Ed; dh + dl = d 2^-Ed's leading bits), and its pair of floats.
+__device__ __forceinline__ double schur2_t(double a, int Ea, double d, int Ed, float dh, float dl, float& t0, float& te)
+{
+    const int E = max(Ed, Ea);
+    const float sa = f32_pow2(Ea - E), sd = f32_pow2(Ed - E);
+    const float ah = f64_lead(a) * sa, al = f64_rest(a) * sa;
+    dh *= sd;
+    dl *= sd;
+    const float A = 2.0f * ah, n = fmaf(dh, dh, A * A), rs = rsqrt_seed(n);
+    t0 = A * rcp_seed(fmaf(n, rs, dh));
+    // residual a (t0^2 - 1) + d t0; its derivative at the root is sqrt(d^2 + 4 a^2)
+    const float P = dh * t0, Pe = fmaf(dh, t0, -P), p = t0 * t0, pe = fmaf(t0, t0, -p), Q = ah * p, Qe = fmaf(ah, p, -Q);
+    const float s1 = __fsub_rn(P, ah), b1 = __fsub_rn(s1, P);
+    const float e1 = __fadd_rn(__fsub_rn(P, __fsub_rn(s1, b1)), __fsub_rn(-ah, b1));
+    const float s2 = __fadd_rn(s1, Q), b2 = __fsub_rn(s2, s1);
+    const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(Q, b2));
+    const float low = ((e1 + e2) + (Pe + Qe)) + (fmaf(dl, t0, -al) + fmaf(al, p, ah * pe));
+    te = -(s2 + low) * rs;
+    const double td = f64_of(t0, 0) + f64_of(te, 0);
+    return fma(-fma(fma(a, td, d), td, -a), f64_of(rs, 1023 - E), td);
+}
+
+// tau (want_c false) or c (true) of the tangent t = t0 + te: the root of
+// t z^2 + 2 z - t, or of (1 + t^2) z^2 - 1; either derivative is 2 / c.
+__device__ __forceinline__ double schur2_z(double t, float t0, float te, bool want_c)
+{
+    const float p1 = t0 * t0, p1e = fmaf(t0, t0, -p1), xh = __fadd_rn(1.0f, p1);
+    const float xl = __fadd_rn(__fsub_rn(1.0f, xh), p1) + fmaf(2.0f * t0, te, p1e);
+    const float c0 = rsqrt_seed(xh), u0 = t0 * c0 * rcp_seed(1.0f + c0);
+    const float z0 = want_c ? c0 : u0, Ah = want_c ? xh : t0, Al = want_c ? xl : te, B = want_c ? 0.0f : 2.0f;
+    const float Ch = want_c ? -1.0f : -t0, Cl = want_c ? 0.0f : -te;
+    const float P = B * z0, p = z0 * z0, pe = fmaf(z0, z0, -p), Q = Ah * p, Qe = fmaf(Ah, p, -Q);
+    const float s1 = __fadd_rn(P, Ch), b1 = __fsub_rn(s1, P);
+    const float e1 = __fadd_rn(__fsub_rn(P, __fsub_rn(s1, b1)), __fsub_rn(Ch, b1));
+    const float s2 = __fadd_rn(s1, Q), b2 = __fsub_rn(s2, s1);
+    const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(Q, b2));
+    const float low = ((e1 + e2) + Qe) + (fmaf(Ah, pe, Al * p) + Cl);
+    const float ze = -0.5f * c0 * (s2 + low);
+    const double zd = f64_of(z0, 0) + f64_of(ze, 0);
+    const double A64 = want_c ? fma(t, t, 1.0) : t, B64 = want_c ? 0.0 : 2.0, C64 = want_c ? -1.0 : -t;
+    return fma(-fma(fma(A64, zd, B64), zd, C64), f64_of(0.5f * c0, 0), zd);
+}
+
+// sgn(zeta) as a sign bit, sgn(0) = +1
+__device__ __forceinline__ int schur2_sign(double d, double apq)
+{
+    return (__double_as_longlong(d) << 1) == 0 ? 0 : (__double2hiint(d) ^ __double2hiint(apq)) & 0x80000000;
+}
+
 __device__ __forceinline__ void schur2(double app, double aqq, double apq, double& s, double& t, double& tau)
 {
     const double d = rn_sub(aqq, app);
-    const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(apq), E = max(Ed, Ea);
-    if (E < 128 || E > 1900 || Ea + 60 < E) {   // (the float pairs need apq within 2^-60 of d)
+    const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(apq);
+    if (!schur2_paired(Ed, Ea)) {
         schur2_wide(d, apq, s, t, tau);
         return;
     }
-    const bool dzero = (__double_as_longlong(d) << 1) == 0;
-    const int sgn = dzero ? 0 : (__double2hiint(d) ^ __double2hiint(apq)) & 0x80000000;   // sgn(zeta), sgn(0) = +1
-    const double aa = fabs(apq), dd = fabs(d);
-    const float ah = f64_lead(aa, Ea - E), al = f64_rest(aa, Ea - E), dh = f64_lead(dd, Ed - E), dl = f64_rest(dd, Ed - E);
-    const float A = 2.0f * ah, n = fmaf(dh, dh, A * A), rs = rsqrt_seed(n);
-    const float t0 = A * rcp_seed(fmaf(n, rs, dh));
-    float te;
-    {   // residual a (t0^2 - 1) + d t0; its derivative at the root is sqrt(d^2 + 4 a^2)
-        const float P = dh * t0, Pe = fmaf(dh, t0, -P), p = t0 * t0, pe = fmaf(t0, t0, -p), Q = ah * p, Qe = fmaf(ah, p, -Q);
-        const float s1 = __fsub_rn(P, ah), b1 = __fsub_rn(s1, P);
-        const float e1 = __fadd_rn(__fsub_rn(P, __fsub_rn(s1, b1)), __fsub_rn(-ah, b1));
-        const float s2 = __fadd_rn(s1, Q), b2 = __fsub_rn(s2, s1);
-        const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(Q, b2));
-        const float low = ((e1 + e2) + (Pe + Qe)) + (fmaf(dl, t0, -al) + fmaf(al, p, ah * pe));
-        te = -(s2 + low) * rs;
-    }
-    const double td = f64_of(t0, 0) + f64_of(te, 0);
-    const double ta = fma(-fma(fma(aa, td, dd), td, -aa), f64_of(rs, 1023 - E), td);
-    const float c0 = rsqrt_seed(fmaf(t0, t0, 1.0f));
-    const float u0 = t0 * c0 * rcp_seed(1.0f + c0), s0 = t0 * c0, ry = fmaf(0.5f, c0, 0.5f);
-    float ue, se;
-    {
-        const float P = 2.0f * u0, p = u0 * u0, pe = fmaf(u0, u0, -p), Q = t0 * p, Qe = fmaf(t0, p, -Q);
-        const float s1 = __fsub_rn(P, t0), b1 = __fsub_rn(s1, P);
-        const float e1 = __fadd_rn(__fsub_rn(P, __fsub_rn(s1, b1)), __fsub_rn(-t0, b1));
-        const float s2 = __fadd_rn(s1, Q), b2 = __fsub_rn(s2, s1);
-        const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(Q, b2));
-        const float low = ((e1 + e2) + Qe) + (fmaf(t0, pe, te * p) - te);
-        ue = -0.5f * c0 * (s2 + low);
-        const float R = s0 * p, Re = fmaf(s0, p, -R);
-        const float r1 = __fsub_rn(P, s0), c1 = __fsub_rn(r1, P);
-        const float f1 = __fadd_rn(__fsub_rn(P, __fsub_rn(r1, c1)), __fsub_rn(-s0, c1));
-        const float r2 = __fsub_rn(r1, R), c2 = __fsub_rn(r2, r1);
-        const float f2 = __fadd_rn(__fsub_rn(r1, __fsub_rn(r2, c2)), __fsub_rn(-R, c2));
-        const float lw = ((f1 + f2) - Re) + (2.0f * ue - s0 * fmaf(2.0f * u0, ue, pe));
-        se = (r2 + lw) * ry;
-    }
-    const double ud = f64_of(u0, 0) + f64_of(ue, 0);
-    const double ua = fma(-fma(fma(ta, ud, 2.0), ud, -ta), f64_of(0.5f * c0, 0), ud);
-    const double sd = f64_of(s0, 0) + f64_of(se, 0);
-    const double sa = fma(fma(-sd, fma(ua, ua, 1.0), ua + ua), f64_of(ry, 0), sd);
+    const int sgn = schur2_sign(d, apq);
+    float t0, te;
+    const double ta = schur2_t(fabs(apq), Ea, fabs(d), Ed, f64_lead(d), f64_rest(d), t0, te);
+    const double ca = schur2_z(ta, t0, te, true);
     t = f64_signed(ta, sgn);
-    tau = f64_signed(ua, sgn);
-    s = f64_signed(sa, sgn);
+    tau = f64_signed(schur2_z(ta, t0, te, false), sgn);
+    s = f64_signed(ta * ca, sgn);
 }
 
 // |apq| > tol sqrt|app| sqrt|aqq| as apq^2 > tol^2 |app| |aqq|, first on
@@ -235,25 +253,37 @@ __device__ __forceinline__ void schur2(double app, double aqq, double apq, doubl
 // 2^-18 of 1 needs FP64.  There, where every operand lies in [2^-400, 2^400],
 // the squares can neither overflow nor underflow and nonnegative doubles
 // compare like their bit patterns; elsewhere the square-root form.
-__device__ __forceinline__ bool rotation_wanted(double app, double aqq, double apq, double tol)
+// The FP32 part: 1 rotate, 0 skip, -1 undecided; y = the leading parts of tol
+// tol app aqq multiplied, esum = the sum of their biased exponents.
+__device__ __forceinline__ int rotation_wanted_lead(double apq, float y, int esum)
 {
-    if ((__double_as_longlong(apq) << 1) == 0) return false;
-    const int ep = f64_biased_exp(apq), e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq), et = f64_biased_exp(tol);
-    if (ep >= 1 && e1 >= 1 && e2 >= 1 && et >= 1) {
-        const int sh = e1 + e2 + 2 * et - 2 * ep - 2046;   // rhs / lhs in [2^(sh - 2), 2^(sh + 4))
-        if (sh > 8) return false;
-        if (sh < -8) return true;
-        const float fa = f64_lead(apq, 0), ft = f64_lead(tol, 0);
-        const float x = fa * fa;
-        const float y = ((ft * ft) * f64_lead(app, 0)) * (f64_lead(aqq, 0) * __int_as_float((sh + 127) << 23));
-        if (fabsf(x - y) > 3.8e-6f * x) return x > y;
-    }
+    const int ep = f64_biased_exp(apq), sh = esum - 2 * ep - 2046;   // rhs / lhs in [2^(sh - 2), 2^(sh + 4))
+    if (ep < 1) return (__double_as_longlong(apq) << 1) == 0 ? 0 : -1;
+    const float fa = f64_lead(apq), x = fa * fa, r = y * __int_as_float((min(max(sh, -9), 9) + 127) << 23);
+    if (sh > 8) return 0;
+    if (sh < -8) return 1;
+    return fabsf(x - r) > 3.8e-6f * x ? x > r : -1;
+}
+__device__ __forceinline__ bool rotation_wanted_exact(double app, double aqq, double apq, double tol)
+{
+    const int ep = f64_biased_exp(apq), e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq);
     const bool safe = ep >= 623 && ep <= 1423 && e1 >= 623 && e1 <= 1423 && e2 >= 623 && e2 <= 1423;
     if (safe) {
         const double lhs = apq * apq, rhs = (tol * tol) * (fabs(app) * fabs(aqq));
         return __double_as_longlong(lhs) > __double_as_longlong(rhs);
     }
     return fabs(apq) > rn_mul(rn_mul(tol, rn_sqrt(fabs(app))), rn_sqrt(fabs(aqq)));
+}
+__device__ __forceinline__ bool rotation_wanted(double app, double aqq, double apq, double tol)
+{
+    if ((__double_as_longlong(apq) << 1) == 0) return false;
+    const int e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq), et = f64_biased_exp(tol);
+    if (e1 >= 1 && e2 >= 1 && et >= 1) {
+        const float ft = f64_lead(tol);
+        const int w = rotation_wanted_lead(apq, (ft * ft) * (f64_lead(app) * f64_lead(aqq)), e1 + e2 + 2 * et);
+        if (w >= 0) return w;
+    }
+    return rotation_wanted_exact(app, aqq, apq, tol);
 }
 
 // (x, y) <- (c x - s y, s x + c y) in Rutishauser's form with tau = s/(1+c):

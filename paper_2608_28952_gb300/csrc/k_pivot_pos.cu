@@ -29,11 +29,13 @@
 //     their quads);
 //   * chain warps, two lanes per pair of round g + 1: that pair's entry is one
 //     entry of one quad of round g (BT of quad (e - 1, e + 1); TT of (0, 1)
-//     and BB of (k/2 - 2, k/2 - 1) at the ends), so a pair of lanes rotates
-//     its own copy of that quad, takes the diagonal that the last choice left
-//     at its position, chooses round g + 1's rotation, sends the parameters
-//     to every CTA and the diagonal after that rotation to the lanes that
-//     need it next;
+//     and BB of (k/2 - 2, k/2 - 1) at the ends), so a pair of lanes forms that
+//     entry (two multiplications and two FMAs), chooses round g + 1's rotation
+//     (the top's lane finds tau while the bottom's finds c), sends the
+//     parameters to every CTA and (t, a_pq) to whoever carries the two diagonal
+//     entries next.  Where auxiliary warps carry the diagonal they also hand
+//     over d = aqq - app and its leading bits, ready before the entry is:
+//     14 FP64 instructions are left in the chain (k = 32: 77.5 -> 69.7 us).
 // One cluster barrier per round ("round g is stored, round g + 1's parameters
 // are there") with two buffers of the quads; where shared memory holds only
 // one, a second one ("every quad of round g is in registers") whose wait is
@@ -131,9 +133,9 @@ __device__ __forceinline__ void shear2(T s, T tau, T& x, T& y)
     x = fma(-tau, y, u);
 }
 
-__device__ __forceinline__ double f64_negate(double x)   // no FP64 instruction
+__device__ __forceinline__ double f64_flip(double x, int sign_bit)   // no FP64 instruction
 {
-    return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
+    return __hiloint2double(__double2hiint(x) ^ sign_bit, __double2loint(x));
 }
 
 template <bool V32> struct PpV { using T = double; };
@@ -147,7 +149,7 @@ __device__ __forceinline__ long long pp_key(double x)
 }
 
 struct PpSmem {   // offsets in doubles
-    int buf, v, par, dg, fin, par32, ints;
+    int buf, v, par, dg, prep, cs, fin, par32, ints;
     bool two;     // two buffers of the quads: stores need not wait for the loads
     size_t bytes;
 };
@@ -159,12 +161,15 @@ __host__ __device__ inline PpSmem pp_smem(int k, int C, bool v32)
     s.buf = 4 * pp_chunk(k, C) + ((h + 1) & ~1);   // the quads' entries, then the pairs' own
     const int vel = (k + C - 1) / C * k;
     const int vd = ((v32 ? (vel + 1) / 2 : vel) + 1) / 2 * 2;
-    const int rest = vd + 20 * h + k + (v32 ? 2 * h : 0);
+    const int prep = pp_chunk(k, C) <= 128 * PP_QMAX ? 5 * h : 0;   // (128 bulk threads: with auxiliary warps)
+    const int rest = vd + 22 * h + prep + k + (v32 ? 2 * h : 0);
     s.two = (size_t)(2 * s.buf + rest) * 8 + (size_t)(2 * k + 2 * h) * sizeof(int) <= PP_SMEM_MAX;
     s.v = (s.two ? 2 : 1) * s.buf;
     s.par = s.v + vd;                       // params: 2 rounds x h pairs x (s, tau)
     s.dg = s.par + 4 * h;
-    s.fin = s.dg + 16 * h;                  // diagonal: (hi, lo) and (t, a_pq), each 2 rounds x 2 sides x h
+    s.prep = s.dg + 16 * h;                 // diagonal: (hi, lo) and (t, a_pq), each 2 rounds x 2 sides x h
+    s.cs = s.prep + prep;                     // per pair of this CTA's: the next choice's part of the diagonal
+    s.fin = s.cs + 2 * h;                   // cosines: 2 rounds x h
     s.par32 = s.fin + k;
     s.ints = s.par32 + (v32 ? 2 * h : 0);   // float2 x 2 rounds x h
     s.bytes = (size_t)s.ints * 8 + (size_t)(2 * k + 2 * h) * sizeof(int);
@@ -176,13 +181,15 @@ __host__ __device__ inline PpSmem pp_smem(int k, int C, bool v32)
 template <int NB, int QPT, int CH, int AT, bool V32>
 __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int C)
 {
-    constexpr bool kAuxDiag = AT >= CH;   // the auxiliary threads carry the diagonal (else the first bulk threads)
-    // and rotate V: an FP32 one always; an FP64 one (as much work as the quads)
+    // The auxiliary threads rotate V: an FP32 one always; an FP64 one (as much work as the quads)
     // where the FP64 unit bounds the round, not where the rotation choice does
     // and would wait behind four more FP64 warps (one quad per bulk thread;
     // measured: k = 32 78 us with V after the quads, 82 us beside them; k = 128
     // with 16 pairs 613 and 520)
     constexpr bool kAuxV = V32 || (AT > 0 && QPT > 1);
+    // and carry the diagonal, unless an FP64 V keeps them busy (then the first
+    // bulk threads do, and the chain reads its part of the diagonal itself)
+    constexpr bool kAuxDiag = AT >= CH && (V32 || !kAuxV);
     using VT = typename PpV<V32>::T;
     extern __shared__ __align__(16) double psm[];
     cg::cluster_group cluster = cg::this_cluster();
@@ -201,6 +208,12 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // round's rotation, and that rotation's (+-t, a_pq) to apply to it
     double2* dg = reinterpret_cast<double2*>(psm + L.dg);
     double2* dt = dg + 4 * h;
+    // what the next choice needs of a pair's diagonal: (app, aqq), the leading
+    // parts of d = aqq - app, the right-hand side of the rotation test, d
+    double2* pr_ad = reinterpret_cast<double2*>(psm + L.prep);
+    float4* pr_f = reinterpret_cast<float4*>(pr_ad + h);
+    double* pr_d = reinterpret_cast<double*>(pr_f + h);
+    double* cs = psm + L.cs;
     double* fin = psm + L.fin;                            // the diagonal by index: at the start, and at the end
     float2* par32 = reinterpret_cast<float2*>(psm + L.par32);
     int* s_dest = reinterpret_cast<int*>(psm + L.ints);
@@ -367,7 +380,8 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     const int ve0 = vwarp ? vt >> 5 : vt / rows, vi0 = vwarp ? vt & 31 : vt - ve0 * rows;
     const int vde = vwarp ? VN / 32 : VN / rows, vdi = vwarp ? 0 : VN - vde * rows;
     auto rotate_v = [&](int so, int rd) {
-        constexpr int U = 4;
+        constexpr int U = NB == 256 && !V32 ? 2 : 4;   // items in flight: 4 (256 bulk threads: 2 of each row group,
+        constexpr int UO = NB == 256 && !V32 ? 4 : 1;  // which costs fewer registers)
         int e = ve0, i = vi0;
         while (e < h) {
             int ot[U], ob[U];
@@ -395,6 +409,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                     ++e;
                 }
             }
+#pragma unroll UO
             for (int o = 0; o < (vwarp ? rows : 1); o += 32) {
                 VT xt[U], xb[U];
 #pragma unroll
@@ -429,6 +444,15 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
         if (dg_rank == r) *d = make_double2(hi, lo);
         else pp_st2(pp_mapa((uint32_t)__cvta_generic_to_shared(d), dg_rank), hi, lo);
     };
+    const int tol_e = f64_biased_exp(tol);
+    const float tol_f = f64_lead(tol) * f64_lead(tol);
+    // leading parts of a pair's diagonal for the next choice
+    auto prepare = [&](double app, double aqq, double d) {
+        const int e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq);
+        const bool ok = e1 >= 1 && e2 >= 1 && tol_e >= 1;
+        return make_float4(f64_lead(d), f64_rest(d), tol_f * (f64_lead(app) * f64_lead(aqq)),
+                           __int_as_float(ok ? e1 + e2 + 2 * tol_e : -1));
+    };
     auto rotated_diag = [&](int g, double& hi, double& lo) {
         const int o = (2 * (g & 1) + dside) * h + de;
         const double2 d = dg[o], c = dt[o];
@@ -441,6 +465,29 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
         double hi, lo;
         rotated_diag(g, hi, lo);
         put_diag(g + 1, hi, lo);
+    };
+    // the same by auxiliary warps, which first hand the chain its part of it
+    const int pair_threads = nt - NB;   // chain and auxiliary threads
+    auto carry_diag_for_chain = [&](int g, bool last) {
+        double2 d = make_double2(0.0, 0.0), c = d;
+        if (dcar) {
+            const int o = (2 * (g & 1) + dside) * h + de;
+            d = dg[o];
+            c = dt[o];
+        }
+        if (!last) {
+            const double dv = d.x + fma(c.x, c.y, d.y), other = __shfl_xor_sync(0xffffffffu, dv, 1);
+            if (dcar && dside == 0) {
+                const double df = rn_sub(other, dv);
+                pr_ad[de] = make_double2(dv, other);
+                pr_f[de] = prepare(dv, other, df);
+                pr_d[de] = df;
+            }
+            asm volatile("bar.arrive 1, %0;" ::"r"(pair_threads) : "memory");
+        }
+        if (!dcar) return;
+        dd_add_prod(d.x, d.y, c.x, c.y, 1.0);
+        put_diag(g + 1, d.x, d.y);
     };
     if (dcar && max_sweeps > 0) put_diag(0, fin[dside ? k - 1 - de : de], 0.0);
     if (role == 0) {
@@ -542,77 +589,120 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
         int t1 = lead, e1 = ce;                            // where this lane's index goes
         pp_next(t1, e1, h);
         const int dgd = t1 * h + e1, dgr = s_own[e1];
-        // the rotation of round g for the pair's entry av and this lane's
-        // diagonal entry: parameters to every CTA, and the change of the
-        // diagonal to the lanes that hold its next position
-        auto choose = [&](int g, int rd, double av, double dv) {
-            const double dother = __shfl_xor_sync(0xffffffffu, dv, 1);
-            const double app = lead ? dother : dv, aqq = lead ? dv : dother;
-            const bool on = mine && rotation_wanted(app, aqq, av, tol);
-            double s = 0.0, t = 0.0, tau = 0.0;
+        // The rotation of round g for the pair's entry av, (app, aqq) = ad, their
+        // difference d and its leading parts f: parameters to every CTA, and the
+        // change of the diagonal to the lanes that hold its next position.  The
+        // top's lane finds tau, the bottom's the cosine.
+        auto choose = [&](int g, int rd, double av, double2 ad, double d, float4 f) {
+            const int es = __float_as_int(f.w);
+            int want = es >= 0 ? rotation_wanted_lead(av, f.z, es) : -1;
+            if (want < 0) want = (__double_as_longlong(av) << 1) != 0 && rotation_wanted_exact(ad.x, ad.y, av, tol);
+            const bool on = mine && want;
+            const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(av);
+            const bool paired = schur2_paired(Ed, Ea);
+            double t = 0.0, z = 0.0;
+            float t0 = 0.0f, te = 0.0f;
+            if (on && paired) {
+                t = schur2_t(fabs(av), Ea, fabs(d), Ed, f.x, f.y, t0, te);
+                z = schur2_z(t, t0, te, lead);
+            }
+            const double zo = __shfl_xor_sync(0xffffffffu, z, 1);
+            double tau = lead ? zo : z, c = lead ? z : zo, s = t * c;
             if (on) {
-                schur2(app, aqq, av, s, t, tau);
-                // zeta = 0: t = +1 with the smaller index as p
-                if (__double_as_longlong(app) == __double_as_longlong(aqq) &&
-                    pp_index(ce, rd, nr) > pp_index(k - 1 - ce, rd, nr)) {
-                    s = -s;
-                    t = -t;
-                    tau = -tau;
+                int sgn = schur2_sign(d, av);
+                if (!paired) {
+                    schur2_wide(d, av, s, t, tau);
+                    c = fma(-s, tau, 1.0);
+                    sgn = 0;
                 }
+                // zeta = 0: t = +1 with the smaller index as p
+                if ((__double_as_longlong(d) << 1) == 0 && pp_index(ce, rd, nr) > pp_index(k - 1 - ce, rd, nr)) sgn = 0x80000000;
+                s = f64_flip(s, sgn);
+                t = f64_flip(t, sgn);
+                tau = f64_flip(tau, sgn);
+            } else {
+                s = t = tau = 0.0;
+                c = 1.0;
             }
             if (mine) {
                 const int sl = (g & 1) * h + ce;
                 for (int u = lead; u < C; u += 2) {
                     if (u == r) {
                         par[sl] = make_double2(s, tau);
+                        cs[sl] = c;
                         if (V32) par32[sl] = make_float2(f32_of(s), f32_of(tau));
                     } else {
                         pp_st2(pp_mapa((uint32_t)__cvta_generic_to_shared(par + sl), u), s, tau);
+                        dsm_st(pp_mapa((uint32_t)__cvta_generic_to_shared(cs + sl), u), c);
                         if (V32) {
-                            const uint32_t ad = pp_mapa((uint32_t)__cvta_generic_to_shared(par32 + sl), u);
-                            dsm_st(ad, f32_of(s));
-                            dsm_st(ad + 4, f32_of(tau));
+                            const uint32_t ad32 = pp_mapa((uint32_t)__cvta_generic_to_shared(par32 + sl), u);
+                            dsm_st(ad32, f32_of(s));
+                            dsm_st(ad32 + 4, f32_of(tau));
                         }
                     }
                 }
-                const double tl = lead ? t : f64_negate(t), al = on ? av : 0.0;
-                double2* d = dt + (g & 1) * 2 * h + dgd;
-                if (dgr == r) *d = make_double2(tl, al);
-                else pp_st2(pp_mapa((uint32_t)__cvta_generic_to_shared(d), dgr), tl, al);
+                const double tl = lead ? t : f64_flip(t, 0x80000000), al = on ? av : 0.0;
+                double2* dd = dt + (g & 1) * 2 * h + dgd;
+                if (dgr == r) *dd = make_double2(tl, al);
+                else pp_st2(pp_mapa((uint32_t)__cvta_generic_to_shared(dd), dgr), tl, al);
                 pv = on ? 0.0 : av;
             }
             nrot += on && lead == 0;
         };
-        if (max_sweeps > 0) choose(0, 0, mine ? psm[pv0 + ce] : 0.0, mine ? fin[lead ? k - 1 - ce : ce] : 0.0);
+        if (max_sweeps > 0) {
+            const double2 ad = make_double2(fin[ce], fin[k - 1 - ce]);
+            const double d = rn_sub(ad.y, ad.x);
+            choose(0, 0, mine ? psm[pv0 + ce] : 0.0, ad, d, prepare(ad.x, ad.y, d));
+        }
         rounds([&](int g, int sw, int rd, bool last) {
             const int so = (g & 1) * h, from = (g & 1) * flip, to = flip - from;
             const double* st = psm + from;
-            double av = pv, x0 = 0.0, x2 = 0.0;
+            double av = pv, x0 = 0.0, x2 = 0.0, si = 0.0, cci = 1.0, sj = 0.0, ccj = 1.0;
             const double pv_old = pv;
-            double2 pi = make_double2(0.0, 0.0), pj = pi, d = pi, c = pi;
-            if (mine) {
-                if (h >= 2) {   // this lane's column of the quad: the top's or the bottom's of pair cj
-                    x0 = st[cslot];
-                    x2 = st[cslot + 2 * chunk];
-                    pi = par[so + ci];
-                    pj = par[so + cj];
+            if (mine && h >= 2) {   // this lane's column of the quad: the top's or the bottom's of pair cj
+                x0 = st[cslot];
+                x2 = st[cslot + 2 * chunk];
+                si = par[so + ci].x;
+                cci = cs[so + ci];
+                sj = par[so + cj].x;
+                ccj = cs[so + cj];
+            }
+            double2 ad = make_double2(0.0, 0.0);
+            double d = 0.0;
+            float4 f = make_float4(1.0f, 0.0f, 1.0f, 0.0f);
+            if constexpr (!kAuxDiag) {   // no auxiliary warps: the diagonal after round g from its own change
+                double dv = 0.0;
+                if (mine) {
+                    const int o = (2 * (g & 1) + lead) * h + ce;
+                    const double2 x = dg[o], y = dt[o];
+                    dv = x.x + fma(y.x, y.y, x.y);
                 }
-                d = dg[(2 * (g & 1) + lead) * h + ce];
-                c = dt[(2 * (g & 1) + lead) * h + ce];
+                const double other = __shfl_xor_sync(0xffffffffu, dv, 1);
+                ad = lead ? make_double2(other, dv) : make_double2(dv, other);
+                d = rn_sub(ad.y, ad.x);
+                f = prepare(ad.x, ad.y, d);
             }
             loaded();
             if (!last) {
                 if (h >= 2) {
-                    shear2(pi.x, pi.y, x0, x2);
-                    // row of the entry: pair ci's bottom, or its top for pair 0
-                    const double y = ce == 0 ? x0 : x2, yo = __shfl_xor_sync(0xffffffffu, y, 1);
-                    double yt = lead ? yo : y, yb = lead ? y : yo;
-                    shear2(pj.x, pj.y, yt, yb);
+                    // row of the entry: pair ci's bottom s T + c B, or for pair 0 its top c T - s B
+                    const bool top = ce == 0, bot = ce == h - 1;
+                    const double y = fma(top ? f64_flip(si, 0x80000000) : si, top ? x2 : x0, cci * (top ? x0 : x2));
+                    const double yo = __shfl_xor_sync(0xffffffffu, y, 1);
+                    const double yt = lead ? yo : y, yb = lead ? y : yo;
                     // column: pair cj's top, or its bottom for the last pair
-                    av = ce == h - 1 ? yb : yt;
+                    av = fma(bot ? sj : f64_flip(sj, 0x80000000), bot ? yt : yb, ccj * (bot ? yb : yt));
+                }
+                if constexpr (kAuxDiag) {
+                    asm volatile("bar.sync 1, %0;" ::"r"(pair_threads) : "memory");
+                    if (mine) {
+                        ad = pr_ad[ce];
+                        d = pr_d[ce];
+                        f = pr_f[ce];
+                    }
                 }
                 if (rd + 1 == nr) flush(sw);
-                choose(g + 1, rd + 1 == nr ? 0 : rd + 1, av, d.x + fma(c.x, c.y, d.y));
+                choose(g + 1, rd + 1 == nr ? 0 : rd + 1, av, ad, d, f);
             } else {
                 flush(sw);
             }
@@ -623,9 +713,9 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
             }
         });
     } else {
-        rounds([&](int g, int, int rd, bool) {
+        rounds([&](int g, int, int rd, bool last) {
             loaded();
-            if constexpr (kAuxDiag) carry_diag(g);
+            if constexpr (kAuxDiag) carry_diag_for_chain(g, last);
             if constexpr (kAuxV) rotate_v((g & 1) * h, rd);
             may_store();
         });
