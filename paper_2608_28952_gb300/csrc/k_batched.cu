@@ -30,7 +30,7 @@ template <typename T>
 __host__ __device__ static size_t core_bytes(int kmax)
 {
     const int half = kmax / 2;
-    return (size_t)4 * half * sizeof(T) + (size_t)kmax * sizeof(T) + (size_t)3 * half * sizeof(int) + 64;
+    return (size_t)4 * half * sizeof(T) + (size_t)kmax * sizeof(T) + (size_t)2 * half * sizeof(int) + 64;
 }
 
 template <typename T>
@@ -38,14 +38,9 @@ __device__ __forceinline__ CoreSmem<T> carve_core(unsigned char* base, int kmax)
 {
     const int half = kmax / 2;
     CoreSmem<T> cs;
-    cs.tau = (T*)base;
-    cs.s = cs.tau + half;
-    cs.t = cs.s + half;
-    cs.apq = cs.t + half;
-    cs.dlo = cs.apq + half;
-    cs.p = (int*)(cs.dlo + kmax);
-    cs.q = cs.p + half;
-    cs.on = cs.q + half;
+    cs.st = (T*)base;
+    cs.dlo = cs.st + 4 * half;
+    cs.pk = (int*)(cs.dlo + kmax);
     return cs;
 }
 
@@ -412,6 +407,38 @@ template cudaError_t launch_batched_svd<double>(const BatchedSvdArgs<double>&, i
 // broadcasts.  Each output is the FMA chain over l = 0..n-1 in order.
 // X may be global (G) or shared (the accumulated V); no tile's rows are read
 // after they are written.  All threads call; blockDim.x is a multiple of 32.
+// Rows r0 .. r0 + tr - 1 of the n columns of X into the tile (columns n ..
+// pad - 1 zero).  A thread keeps one row and steps over the columns (nt / 64 at a
+// time), four loads in flight: dealing the elements by idx % tr and idx / tr
+// cost two integer divisions each.
+template <typename T>
+__device__ __forceinline__ void svd_load_tile(const T* X, size_t ldx, int r0, int tr, int n, int pad, T* tile)
+{
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (nt % kSvdTileRows) {
+        for (int idx = tid; idx < tr * pad; idx += nt) {
+            const int rr = idx % tr, c = idx / tr;
+            tile[c * kSvdTileLd + rr] = c < n ? X[(size_t)(r0 + rr) + ldx * c] : T(0);
+        }
+        return;
+    }
+    const int rr = tid % kSvdTileRows, step = nt / kSvdTileRows;
+    if (rr >= tr) return;
+    const T* x = X + r0 + rr;
+    T* t = tile + rr;
+    for (int c = tid / kSvdTileRows; c < pad; c += 4 * step) {
+        T v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int cc = c + u * step;
+            v[u] = cc < n ? x[ldx * cc] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (c + u * step < pad) t[(c + u * step) * kSvdTileLd] = v[u];
+    }
+}
+
 template <typename T>
 __device__ void svd_rotate_rows(T* X, size_t ldx, int rows, int n, int k, const T* Vh, const int* dest, T* tile)
 {
@@ -420,10 +447,7 @@ __device__ void svd_rotate_rows(T* X, size_t ldx, int rows, int n, int k, const 
     const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
     for (int r0 = 0; r0 < rows; r0 += kSvdTileRows) {
         const int tr = min(kSvdTileRows, rows - r0);
-        for (int idx = tid; idx < tr * n; idx += nt) {
-            const int rr = idx % tr, c = idx / tr;
-            tile[c * kSvdTileLd + rr] = X[(size_t)(r0 + rr) + ldx * c];
-        }
+        svd_load_tile(X, ldx, r0, tr, n, n, tile);
         __syncthreads();
         for (int jc = 0; jc < n; jc += nw * CT) {
             T acc0[CT], acc1[CT];
@@ -486,9 +510,9 @@ __global__ void k_batched_svd_tiled(BatchedSvdArgs<T> a, int kq)
         const size_t ldg = (size_t)a.ldg[mat];
         for (int idx = tid; idx < k * k; idx += nt) Vacc[idx] = (idx % k == idx / k) ? T(1) : T(0);
         int bad = 0;
-        for (int idx = tid; idx < m * n; idx += nt) {
-            if (!isfinite(G[(size_t)(idx % m) + ldg * (idx / m)])) bad = 1;
-        }
+        for (int c = tid >> 5; c < n; c += nt >> 5)
+            for (int r = tid & 31; r < m; r += 32)
+                if (!isfinite(G[r + ldg * c])) bad = 1;
         if (bad) atomicExch(&s_bad, 1);
         __syncthreads();
         const bool nonfinite = s_bad != 0;
@@ -515,10 +539,7 @@ __global__ void k_batched_svd_tiled(BatchedSvdArgs<T> a, int kq)
                     for (int y = 0; y < 4; ++y) acc[x][y] = T(0);
                 for (int r0 = 0; r0 < m; r0 += kSvdTileRows) {
                     const int tr = min(kSvdTileRows, m - r0);
-                    for (int idx = tid; idx < tr * 4 * nb4; idx += nt) {
-                        const int rr = idx % tr, c = idx / tr;
-                        tile[c * kSvdTileLd + rr] = c < n ? G[(size_t)(r0 + rr) + ldg * c] : T(0);
-                    }
+                    svd_load_tile(G, ldg, r0, tr, n, 4 * nb4, tile);
                     __syncthreads();
                     if (own) {
                         const T* ti = tile + 4 * bi * kSvdTileLd;
@@ -605,10 +626,7 @@ __global__ void k_batched_svd_tiled(BatchedSvdArgs<T> a, int kq)
         __syncthreads();
         for (int r0 = 0; r0 < m; r0 += kSvdTileRows) {
             const int tr = min(kSvdTileRows, m - r0);
-            for (int idx = tid; idx < tr * n; idx += nt) {
-                const int rr = idx % tr, c = idx / tr;
-                tile[c * kSvdTileLd + rr] = G[(size_t)(r0 + rr) + ldg * c];
-            }
+            svd_load_tile(G, ldg, r0, tr, n, n, tile);
             __syncthreads();
             for (int j = tid; j < n; j += nt) {
                 T s = nrm[j];
@@ -630,14 +648,12 @@ __global__ void k_batched_svd_tiled(BatchedSvdArgs<T> a, int kq)
         // permute / scale U in place, one staged row tile at a time; V from Vacc
         for (int r0 = 0; r0 < m; r0 += kSvdTileRows) {
             const int tr = min(kSvdTileRows, m - r0);
-            for (int idx = tid; idx < tr * n; idx += nt) {
-                const int rr = idx % tr, c = idx / tr;
-                tile[c * kSvdTileLd + rr] = G[(size_t)(r0 + rr) + ldg * c];
-            }
+            svd_load_tile(G, ldg, r0, tr, n, n, tile);
             __syncthreads();
-            for (int idx = tid; idx < tr * n; idx += nt) {
-                const int rr = idx % tr, j = idx / tr;
-                G[(size_t)(r0 + rr) + ldg * s_dest[j]] = nrm[j] > T(0) ? tile[j * kSvdTileLd + rr] / nrm[j] : T(0);
+            for (int j = tid >> 5; j < n; j += nt >> 5) {   // a warp per column
+                const T nj = nrm[j];
+                T* g = G + r0 + ldg * s_dest[j];
+                for (int rr = tid & 31; rr < tr; rr += 32) g[rr] = nj > T(0) ? tile[j * kSvdTileLd + rr] / nj : T(0);
             }
             __syncthreads();
         }

@@ -260,15 +260,10 @@ __global__ void __launch_bounds__(PIV_T) k_pivot(PivotArgs a)
     VT* V = reinterpret_cast<VT*>(Ap + ntp);
     double* tail = smem;
     CoreSmem<double> cs;
-    cs.tau = tail;
-    cs.s = cs.tau + half;
-    cs.t = cs.s + half;
-    cs.apq = cs.t + half;
-    cs.dlo = cs.apq + half;
-    cs.p = (int*)(cs.dlo + k);
-    cs.q = cs.p + half;
-    cs.on = cs.q + half;
-    unsigned* quad = (unsigned*)(cs.on + half);
+    cs.st = tail;
+    cs.dlo = cs.st + 4 * half;
+    cs.pk = (int*)(cs.dlo + k);
+    unsigned* quad = (unsigned*)(cs.pk + 2 * half);
     __shared__ int s_cnt;
     cs.cnt = &s_cnt;
     __shared__ double s_red[PIV_T / 32];
