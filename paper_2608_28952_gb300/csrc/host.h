@@ -103,6 +103,33 @@ struct PhaseEvents {
     }
 };
 
+// A low-priority stream beside the caller's, with the events that fork from it
+// and join it again.  Destroyed only after its work is done.
+struct SideStream {
+    cudaStream_t s = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    bool open()
+    {
+        int lo = 0, hi = 0;
+        if (cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
+            cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, lo) == cudaSuccess &&
+            cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess)
+            return true;
+        cudaGetLastError();
+        return false;
+    }
+    ~SideStream()
+    {
+        if (s) {
+            cudaStreamSynchronize(s);
+            cudaStreamDestroy(s);
+        }
+        if (fork) cudaEventDestroy(fork);
+        if (join) cudaEventDestroy(join);
+    }
+};
+
 // A captured sweep, replayed on the caller's stream.
 struct SweepGraph {
     cudaGraphExec_t exec = nullptr;
@@ -118,8 +145,11 @@ struct SweepGraph {
 template <class F>
 inline bool capture(SweepGraph& g, F body)
 {
+    // the highest priority: a sweep's own kernels go before those of a SideStream
     cudaStream_t cs;
-    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
+    int lo = 0, hi = 0;
+    if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&cs, cudaStreamNonBlocking, hi) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -222,6 +252,7 @@ struct EvdState {
     int* atab = nullptr;
     unsigned char* qimg = nullptr;
     int* qexp = nullptr;
+    SideStream* side = nullptr;   // their images are made here, beside the pivot solves
     // pivot_order == 2: the per-pair QRCP scratch of the pivoting step
     double* qrws = nullptr;
     // emulated products: balance by the diagonal (relative stop criterion)

@@ -234,7 +234,9 @@ struct EmuUpdArgs {
     unsigned char* qimg = nullptr;
     int* qexp = nullptr;
 };
-cudaError_t launch_emu_update(const EmuUpdArgs& a, cudaStream_t s);
+// operands: make the stage-1 operands' images too (else launch_emu_operands has)
+cudaError_t launch_emu_update(const EmuUpdArgs& a, bool operands, cudaStream_t s);
+cudaError_t launch_emu_operands(const EmuUpdArgs& a, bool skip, cudaStream_t s);
 size_t emu_update_vimg_bytes(int npairs, int k);
 size_t emu_update_vexp_ints(int npairs, int k);
 size_t emu_update_aimg_bytes(int npairs, int k);

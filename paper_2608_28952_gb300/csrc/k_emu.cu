@@ -720,17 +720,42 @@ __global__ void __launch_bounds__(E_T) k_emu_slice_v(const double* __restrict__ 
 
 // Row scales of the stage-1 A operands: out[e][i] = 1 + the largest exponent
 // of X(i, P_e) over the 2b columns of pair e (0 when all are zero), for the
-// rows i < rows of X (the working A, or Q).  Thread = row (coalesced).
-__global__ void k_emu_rowexp(int rows, const double* __restrict__ X, int ld, const int2* __restrict__ pairs,
-                             int b, int* __restrict__ out)
+// rows i < rows of X (the working A, or Q: blockIdx.z).  A warp takes 32 rows
+// (coalesced) and every eighth column, eight loads in flight (one thread
+// walking a row's 2b columns was bound by latency: n = 2048, b = 64: 26 us each
+// for A and Q).
+struct RowExpArgs {
+    int rows[2];
+    const double* X[2];
+    int ld[2];
+    int* out[2];
+};
+__global__ void __launch_bounds__(256) k_emu_rowexp(RowExpArgs a, const int2* __restrict__ pairs, int b)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, e = blockIdx.y;
-    if (i >= rows) return;
+    __shared__ int red[8][32];
+    const int z = blockIdx.z, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int rows = a.rows[z], ld = a.ld[z], i = blockIdx.x * 32 + lane, e = blockIdx.y;
+    const double* X = a.X[z];
     int I, J;
     eentry(pairs, e, I, J);
     int mx = -1100;
-    for (int x = 0; x < 2 * b; ++x) mx = max(mx, exp2_of(X[i + (size_t)ld * emap(I, J, b, x)]));
-    out[(size_t)e * rows + i] = mx <= -1100 ? 0 : mx + 1;
+    if (i < rows)
+        for (int x0 = w; x0 < 2 * b; x0 += 64) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int x = x0 + 8 * u;
+                v[u] = x < 2 * b ? X[i + (size_t)ld * emap(I, J, b, x)] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mx = max(mx, exp2_of(v[u]));
+        }
+    red[w][lane] = mx;
+    __syncthreads();
+    if (w == 0 && i < rows) {
+        for (int u = 1; u < 8; ++u) mx = max(mx, red[u][lane]);
+        a.out[z][(size_t)e * rows + i] = mx <= -1100 ? 0 : mx + 1;
+    }
 }
 
 // The slices of the stage-1 A operands, once per step.  mode 0: pair-block
@@ -758,7 +783,7 @@ __global__ void __launch_bounds__(E_T) k_emu_slice_ops(int mode, const double* _
         eentry(pairs, item, I2, J2);
         eK = item;
     }
-    if (rot[eK] == 0) return;
+    if (rot && rot[eK] == 0) return;
     const int nrow = mode == 0 ? k : rows;
     const int grow = r < nrow ? (mode == 0 ? emap(I1, J1, b, r) : r) : -1;
     const size_t sb = (size_t)R * EK * 2;
@@ -1113,7 +1138,39 @@ size_t emu_update_qimg_bytes(int npairs, int k, int qrows)
     return (size_t)npairs * ((k + EK - 1) / EK) * ENS * emu_img_slice_bytes(qrows);
 }
 
-cudaError_t launch_emu_update(const EmuUpdArgs& a, cudaStream_t s)
+// The images of the stage-1 operands, A's pair-blocks and Q's column pairs:
+// they need nothing of the step's pivot solves, and may run beside them (then
+// without `skip`, which leaves out what the update will only copy).
+cudaError_t launch_emu_operands(const EmuUpdArgs& a, bool skip, cudaStream_t s)
+{
+    const UpdateArgs& u = a.u;
+    if (!a.vimg || u.npairs <= 0) return cudaSuccess;
+    const int nchk = (u.k + EK - 1) / EK, npb = u.npairs * (u.npairs - 1) / 2;
+    const bool A = a.aimg && !a.balance && npb > 0, Q = a.qimg && u.Qin;
+    RowExpArgs r{};
+    int nz = 0, most = 0;
+    auto add = [&](int rows, const double* X, int ld, int* out) {
+        r.rows[nz] = rows;
+        r.X[nz] = X;
+        r.ld[nz] = ld;
+        r.out[nz++] = out;
+        most = rows > most ? rows : most;
+    };
+    if (A) add(u.lda, u.Ain, u.lda, a.atab);
+    if (Q) add(u.qrows, u.Qin, u.ldq, a.qexp);
+    if (!nz) return cudaSuccess;
+    k_emu_rowexp<<<dim3((most + 31) / 32, u.npairs, nz), 256, 0, s>>>(r, u.pairs, u.b);
+    const int* rot = skip ? u.rot : nullptr;
+    if (A)
+        k_emu_slice_ops<<<dim3(nchk, emu_img_rows(u.k) / 64, npb), E_T, 0, s>>>(
+            0, u.Ain, u.lda, u.lda, u.pairs, rot, u.b, u.k, a.atab, emu_img_rows(u.k), a.aimg);
+    if (Q)
+        k_emu_slice_ops<<<dim3(nchk, emu_img_rows(u.qrows) / 64, u.npairs), E_T, 0, s>>>(
+            1, u.Qin, u.ldq, u.qrows, u.pairs, rot, u.b, u.k, a.qexp, emu_img_rows(u.qrows), a.qimg);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_emu_update(const EmuUpdArgs& a, bool operands, cudaStream_t s)
 {
     const UpdateArgs& u = a.u;
     const int nmt = (u.k + EM - 1) / EM, nnt = (u.k + EN - 1) / EN;
@@ -1123,18 +1180,7 @@ cudaError_t launch_emu_update(const EmuUpdArgs& a, cudaStream_t s)
         k_emu_slice_v<<<dim3((u.k + EK - 1) / EK, u.npairs), E_T, 0, s>>>(u.V, u.rot, u.k, a.vexp, a.vimg);
         cudaError_t e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;
-        const int nchk = (u.k + EK - 1) / EK;
-        const int npb = u.npairs * (u.npairs - 1) / 2;
-        if (a.aimg && !a.balance && npb > 0) {   // the pair-blocks of A, sliced once
-            k_emu_rowexp<<<dim3((u.lda + 255) / 256, u.npairs), 256, 0, s>>>(u.lda, u.Ain, u.lda, u.pairs, u.b, a.atab);
-            k_emu_slice_ops<<<dim3(nchk, emu_img_rows(u.k) / 64, npb), E_T, 0, s>>>(
-                0, u.Ain, u.lda, u.lda, u.pairs, u.rot, u.b, u.k, a.atab, emu_img_rows(u.k), a.aimg);
-        }
-        if (a.qimg && u.Qin) {   // the column pairs of Q, sliced once
-            k_emu_rowexp<<<dim3((u.qrows + 255) / 256, u.npairs), 256, 0, s>>>(u.qrows, u.Qin, u.ldq, u.pairs, u.b, a.qexp);
-            k_emu_slice_ops<<<dim3(nchk, emu_img_rows(u.qrows) / 64, u.npairs), E_T, 0, s>>>(
-                1, u.Qin, u.ldq, u.qrows, u.pairs, u.rot, u.b, u.k, a.qexp, emu_img_rows(u.qrows), a.qimg);
-        }
+        if (operands && (e0 = launch_emu_operands(a, true, s)) != cudaSuccess) return e0;
         if ((e0 = cudaGetLastError()) != cudaSuccess) return e0;
     }
     const int npb = u.npairs * (u.npairs - 1) / 2;
