@@ -57,8 +57,18 @@ extern "C" const char* jacobi_status_string(int status)
 // ============================================================================ EVD (FP64)
 namespace jac {
 
+// Q's update of the last step, which the side stream still owes.
+static cudaError_t update_q_pending(EvdState& E)
+{
+    if (!E.pending) return cudaSuccess;
+    E.pending = false;
+    const cudaError_t e = E.T64 ? launch_emu_products(E.pending_q, UPD_Q, E.side->s)
+                                : launch_update_evd(E.pending_q.u, UPD_Q, E.side->s);
+    return e != cudaSuccess ? e : cudaEventRecord(E.side->done[E.pending_cur], E.side->s);
+}
+
 static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, double inner_tol,
-                               int inner_max, int order, cudaEvent_t mid = nullptr)
+                               int inner_max, int order, cudaEvent_t mid = nullptr, int first = 0)
 {
     const int np_s = E.ord.dev_per_step, p0 = s * np_s;
     PivotArgs pa{};
@@ -71,8 +81,8 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
     pa.npairs = np_s;
     pa.b = E.b;
     pa.k = E.k;
-    pa.V = E.Vb;
-    pa.rot = E.rot;
+    pa.V = E.Vb[cur];
+    pa.rot = E.rot[cur];
     pa.relmax = nullptr;
     pa.tol_rel = inner_tol;
     pa.max_sweeps = inner_max;
@@ -93,25 +103,72 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
     ua.npairs = np_s;
     ua.b = E.b;
     ua.k = E.k;
-    ua.V = E.Vb;
-    ua.rot = E.rot;
+    ua.V = E.Vb[cur];
+    ua.rot = E.rot[cur];
     ua.cnt = E.cnt;
-    EmuUpdArgs ea{ua, E.T64, E.err, E.balance, E.vimg, E.vexp, E.aimg, E.atab, E.qimg, E.qexp};
-    // The images of A's and Q's operands need nothing of the pivot solves: made
-    // beside them, on the SMs that the pivots' clusters leave free (n = 2048, b =
-    // 64: 96 of 152 SMs pivot for 0.5 ms; the images take 0.09 ms of all).
-    const bool beside = E.T64 && E.side;
+    EmuUpdArgs ea{ua, E.T64, E.err, E.balance, E.vimg[cur], E.vexp[cur], E.aimg, E.atab, E.qimg, E.qexp};
     cudaError_t e;
-    if (beside && (e = cudaEventRecord(E.side->fork, cs)) != cudaSuccess) return e;
+    if (!E.side) {
+        if ((e = launch_pivot(pa, E.pcl, cs)) != cudaSuccess) return e;
+        if (mid && (e = cudaEventRecordWithFlags(mid, cs, cudaEventRecordExternal)) != cudaSuccess) return e;
+        if (!E.T64) return launch_update_evd(ua, UPD_A | UPD_Q, cs);
+        if ((e = launch_emu_transforms(ea, cs)) != cudaSuccess) return e;
+        if ((e = launch_emu_operands(ea, UPD_A | UPD_Q, true, cs)) != cudaSuccess) return e;
+        return launch_emu_products(ea, UPD_A | UPD_Q, cs);
+    }
+    // The pivot solves' clusters leave SMs free (n = 2048, b = 64: 56 of 152 for
+    // 0.5 ms), and what the next step's pivots need is A alone.  So beside them
+    // a low-priority stream makes the images of A's operands (emulated
+    // products; they need nothing of the pivots) and updates Q by the last
+    // step's transforms, which are kept by step parity.  Q's update is held back
+    // until the next pivots have had 4 us to start: begun any sooner, and even
+    // at the same moment, it fills every SM, and a cluster waits for SMs that
+    // are empty (n = 1000, b = 32: the pivots of a step 157 -> 257 us).  n = 1000,
+    // b = 32 127.5 -> 100 ms, b = 16 141.5 -> 108, n = 2000, b = 64 -7 %; FP64_EMU n
+    // = 1024, b = 32 92.7 -> 77.3, n = 2048, b = 64 281 -> 236, n = 4096 -10 %.
+    pa.alone = 1;
+    SideStream& sd = *E.side;
+    if (first >= 2 && ua.Qin && (e = cudaStreamWaitEvent(cs, sd.done[cur], 0)) != cudaSuccess) return e;
+    if ((e = cudaEventRecord(sd.fork, cs)) != cudaSuccess) return e;
     if ((e = launch_pivot(pa, E.pcl, cs)) != cudaSuccess) return e;
     if (mid && (e = cudaEventRecordWithFlags(mid, cs, cudaEventRecordExternal)) != cudaSuccess) return e;
-    if (beside && ((e = cudaStreamWaitEvent(E.side->s, E.side->fork, 0)) != cudaSuccess ||
-                   (e = launch_emu_operands(ea, false, E.side->s)) != cudaSuccess ||
-                   (e = cudaEventRecord(E.side->join, E.side->s)) != cudaSuccess))
+    if ((e = cudaStreamWaitEvent(sd.s, sd.fork, 0)) != cudaSuccess) return e;
+    if (E.T64 && ((e = launch_emu_operands(ea, UPD_A, false, sd.s)) != cudaSuccess ||
+                  (e = cudaEventRecord(sd.join, sd.s)) != cudaSuccess))
         return e;
-    if (beside && (e = cudaStreamWaitEvent(cs, E.side->join, 0)) != cudaSuccess) return e;
-    if (E.T64) return launch_emu_update(ea, !beside, cs);
-    return launch_update_evd(ua, cs);
+    if (E.pending && (e = launch_pause(4000, sd.s)) != cudaSuccess) return e;
+    if ((e = update_q_pending(E)) != cudaSuccess) return e;
+    if (E.T64 && ((e = launch_emu_operands(ea, UPD_Q, false, sd.s)) != cudaSuccess ||
+                  (e = launch_emu_transforms(ea, cs)) != cudaSuccess ||
+                  (e = cudaStreamWaitEvent(cs, sd.join, 0)) != cudaSuccess))
+        return e;
+    e = E.T64 ? launch_emu_products(ea, UPD_A, cs) : launch_update_evd(ua, UPD_A, cs);
+    E.pending = ua.Qin != nullptr;
+    E.pending_q = ea;
+    E.pending_cur = cur;
+    return e;
+}
+
+// Whether the pivot solves leave SMs for a side stream's kernels, and those are
+// worth the events (n = 256: 12.64 ms without, 12.8 with them; n = 500: 33.3 and
+// 31.4).
+static bool sms_left(const EvdState& E)
+{
+    int dev = 0, sms = 0;
+    return E.np >= 384 && cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           E.ord.dev_per_step * E.pcl < sms;
+}
+
+// The caller's stream waits for all that the side stream still does.
+static cudaError_t join_side(EvdState& E, cudaStream_t cs)
+{
+    if (!E.side) return cudaSuccess;
+    cudaError_t e;
+    if ((e = cudaEventRecord(E.side->fork, cs)) != cudaSuccess || (e = cudaStreamWaitEvent(E.side->s, E.side->fork, 0)) != cudaSuccess ||
+        (e = update_q_pending(E)) != cudaSuccess || (e = cudaEventRecord(E.side->join, E.side->s)) != cudaSuccess)
+        return e;
+    return cudaStreamWaitEvent(cs, E.side->join, 0);
 }
 
 SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double target,
@@ -124,21 +181,22 @@ SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double
     int sw = sweep0;
     PhaseEvents pe(2 * (size_t)E.ord.S + 1);
     SideStream side;
-    E.side = E.aimg && side.open() ? &side : nullptr;
+    E.side = (E.aimg || E.Qw[0]) && sms_left(E) && side.open() ? &side : nullptr;
     for (; sw < p.max_sweeps; ++sw) {
         const int start = cur;
         auto body = [&](cudaStream_t cs) -> bool {
             int c = start;
             if (cudaEventRecordWithFlags(pe.ev[0], cs, cudaEventRecordExternal) != cudaSuccess) return false;
+            E.pending = false;
             for (int si = 0; si < E.ord.S; ++si) {
                 if (launch_step(E, si, c, cs, p.inner_tol, p.inner_max_sweeps, p.pivot_order,
-                                pe.ev[2 * si + 1]) != cudaSuccess)
+                                pe.ev[2 * si + 1], si) != cudaSuccess)
                     return false;
                 if (cudaEventRecordWithFlags(pe.ev[2 * si + 2], cs, cudaEventRecordExternal) != cudaSuccess) return false;
                 c ^= 1;
             }
-            return launch_offnorm(E.np, E.Aw[c], E.partial, E.ticket, E.result, use_rel, cs) ==
-                   cudaSuccess;
+            return launch_offnorm(E.np, E.Aw[c], E.partial, E.ticket, E.result, use_rel, cs) == cudaSuccess &&
+                   join_side(E, cs) == cudaSuccess;
         };
         if (!tried[start]) {
             tried[start] = true;
@@ -201,8 +259,10 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
         E.Aw[1] = ws.get<double>(np2);
         E.Qw[0] = vec ? ws.get<double>(np2) : nullptr;
         E.Qw[1] = vec ? ws.get<double>(np2) : nullptr;
-        E.Vb = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
-        E.rot = ws.get<int>(E.ord.max_pairs);
+        for (int i = 0; i < 2; ++i) {
+            E.Vb[i] = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
+            E.rot[i] = ws.get<int>(E.ord.max_pairs);
+        }
         const size_t gsz = pivot_gscratch_doubles(E.k);
         E.gscratch = gsz ? ws.get<double>(gsz * E.ord.max_pairs) : nullptr;
         E.dpairs = ws.get<int2>(E.ord.dev_pairs.size() / 2);
@@ -217,8 +277,10 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
             E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, E.k));
             E.err = ws.get<int>(1);
             if (emu_image_wanted()) {
-                E.vimg = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
-                E.vexp = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
+                for (int i = 0; i < 2; ++i) {
+                    E.vimg[i] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
+                    E.vexp[i] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
+                }
                 if (p.conv != JACOBI_CONV_REL) {   // (balanced products slice per tile)
                     E.aimg = ws.get<unsigned char>(emu_update_aimg_bytes(E.ord.dev_per_step, E.k));
                     E.atab = ws.get<int>((size_t)E.ord.dev_per_step * E.np);
@@ -730,8 +792,10 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
         E.Aw[1] = ws.get<double>(np2);
         E.Qw[0] = Q ? ws.get<double>(np2) : nullptr;
         E.Qw[1] = Q ? ws.get<double>(np2) : nullptr;
-        E.Vb = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
-        E.rot = ws.get<int>(E.ord.max_pairs);
+        for (int i = 0; i < 1; ++i) {
+            E.Vb[i] = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
+            E.rot[i] = ws.get<int>(E.ord.max_pairs);
+        }
         const size_t gsz = pivot_gscratch_doubles(E.k);
         E.gscratch = gsz ? ws.get<double>(gsz * E.ord.max_pairs) : nullptr;
         E.dpairs = ws.get<int2>(E.ord.dev_pairs.size() / 2);
@@ -742,8 +806,10 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
             E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, E.k));
             E.err = ws.get<int>(1);
             if (emu_image_wanted()) {
-                E.vimg = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
-                E.vexp = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
+                for (int i = 0; i < 1; ++i) {
+                    E.vimg[i] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
+                    E.vexp[i] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
+                }
                 if (p.conv != JACOBI_CONV_REL) {   // (balanced products slice per tile)
                     E.aimg = ws.get<unsigned char>(emu_update_aimg_bytes(E.ord.dev_per_step, E.k));
                     E.atab = ws.get<int>((size_t)E.ord.dev_per_step * E.np);
@@ -771,8 +837,9 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
                                    cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
         SideStream side;
-        E.side = E.aimg && side.open() ? &side : nullptr;
-        if (launch_step(E, step, 0, s, p.inner_tol, p.inner_max_sweeps, p.pivot_order) != cudaSuccess)
+        E.side = E.aimg && sms_left(E) && side.open() ? &side : nullptr;
+        if (launch_step(E, step, 0, s, p.inner_tol, p.inner_max_sweeps, p.pivot_order) != cudaSuccess ||
+            join_side(E, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
         if (cudaMemcpy2DAsync(A, (size_t)lda * 8, E.Aw[1], (size_t)np * 8, (size_t)np * 8, np,
                               cudaMemcpyDeviceToDevice, s) != cudaSuccess)

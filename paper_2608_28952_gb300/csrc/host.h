@@ -107,17 +107,16 @@ struct PhaseEvents {
 // and join it again.  Destroyed only after its work is done.
 struct SideStream {
     cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr, done[2] = {nullptr, nullptr};   // done: Q's update, by step parity
     bool open()
     {
         int lo = 0, hi = 0;
-        if (cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
-            cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, lo) == cudaSuccess &&
-            cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
-            cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess)
-            return true;
-        cudaGetLastError();
-        return false;
+        bool ok = cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
+                  cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, lo) == cudaSuccess;
+        for (cudaEvent_t* e : {&fork, &join, &done[0], &done[1]})
+            ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+        if (!ok) cudaGetLastError();
+        return ok;
     }
     ~SideStream()
     {
@@ -125,8 +124,8 @@ struct SideStream {
             cudaStreamSynchronize(s);
             cudaStreamDestroy(s);
         }
-        if (fork) cudaEventDestroy(fork);
-        if (join) cudaEventDestroy(join);
+        for (cudaEvent_t e : {fork, join, done[0], done[1]})
+            if (e) cudaEventDestroy(e);
     }
 };
 
@@ -233,8 +232,8 @@ struct EvdState {
     int2* dpairs;
     double* Aw[2];
     double* Qw[2];
-    double* Vb;
-    int* rot;
+    double* Vb[2];   // by the step's parity (cur): Q's update reads one while the next pivots write the other
+    int* rot[2];
     double* gscratch;
     double* partial;
     unsigned* ticket;
@@ -245,14 +244,17 @@ struct EvdState {
     double* T64 = nullptr;
     int* err = nullptr;
     // the step's V sliced once (bf16 digit images) and its column scales
-    unsigned char* vimg = nullptr;
-    int* vexp = nullptr;
+    unsigned char* vimg[2] = {nullptr, nullptr};
+    int* vexp[2] = {nullptr, nullptr};
     // and the step's stage-1 operands (A's pair-blocks, Q's column pairs)
     unsigned char* aimg = nullptr;
     int* atab = nullptr;
     unsigned char* qimg = nullptr;
     int* qexp = nullptr;
-    SideStream* side = nullptr;   // their images are made here, beside the pivot solves
+    SideStream* side = nullptr;   // what runs beside the pivot solves: those images, Q's update
+    bool pending = false;         // Q's update of the last step is still to be launched there
+    EmuUpdArgs pending_q{};
+    int pending_cur = 0;
     // pivot_order == 2: the per-pair QRCP scratch of the pivoting step
     double* qrws = nullptr;
     // emulated products: balance by the diagonal (relative stop criterion)

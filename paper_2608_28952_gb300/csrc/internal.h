@@ -88,6 +88,7 @@ struct PivotArgs {
     int n_real;                // rows/columns >= n_real are zero padding
     double* gscratch;          // k > 128 with one CTA per pair: per-pair global scratch (packed A + V)
     double* qrws;              // order == 2: per-pair QRCP scratch, b x k doubles each
+    int alone;                 // keep other kernels' CTAs off the SMs that solve pivots (they run beside these)
     DevCounters* cnt;
 };
 // with C CTAs per pair (C from pivot_cluster_size, or 1)
@@ -108,7 +109,10 @@ struct UpdateArgs {
     const double* V; const int* rot;
     DevCounters* cnt;
 };
-cudaError_t launch_update_evd(const UpdateArgs& a, cudaStream_t s);
+cudaError_t launch_pause(int ns, cudaStream_t s);
+// parts of an update: A's pair-blocks, Q's column pairs
+constexpr int UPD_A = 1, UPD_Q = 2;
+cudaError_t launch_update_evd(const UpdateArgs& a, int parts, cudaStream_t s);
 
 // One-sided update: G'(:,P) = G(:,P) V_P (m rows) and V'(:,P) = V(:,P) V_P.
 struct ColUpdateArgs {
@@ -234,9 +238,11 @@ struct EmuUpdArgs {
     unsigned char* qimg = nullptr;
     int* qexp = nullptr;
 };
-// operands: make the stage-1 operands' images too (else launch_emu_operands has)
-cudaError_t launch_emu_update(const EmuUpdArgs& a, bool operands, cudaStream_t s);
-cudaError_t launch_emu_operands(const EmuUpdArgs& a, bool skip, cudaStream_t s);
+// In this order: the images of the stage-1 operands (skip: only what the
+// update multiplies; they need nothing of the pivot solves), of V, the products.
+cudaError_t launch_emu_operands(const EmuUpdArgs& a, int parts, bool skip, cudaStream_t s);
+cudaError_t launch_emu_transforms(const EmuUpdArgs& a, cudaStream_t s);
+cudaError_t launch_emu_products(const EmuUpdArgs& a, int parts, cudaStream_t s);
 size_t emu_update_vimg_bytes(int npairs, int k);
 size_t emu_update_vexp_ints(int npairs, int k);
 size_t emu_update_aimg_bytes(int npairs, int k);

@@ -1141,12 +1141,12 @@ size_t emu_update_qimg_bytes(int npairs, int k, int qrows)
 // The images of the stage-1 operands, A's pair-blocks and Q's column pairs:
 // they need nothing of the step's pivot solves, and may run beside them (then
 // without `skip`, which leaves out what the update will only copy).
-cudaError_t launch_emu_operands(const EmuUpdArgs& a, bool skip, cudaStream_t s)
+cudaError_t launch_emu_operands(const EmuUpdArgs& a, int parts, bool skip, cudaStream_t s)
 {
     const UpdateArgs& u = a.u;
     if (!a.vimg || u.npairs <= 0) return cudaSuccess;
     const int nchk = (u.k + EK - 1) / EK, npb = u.npairs * (u.npairs - 1) / 2;
-    const bool A = a.aimg && !a.balance && npb > 0, Q = a.qimg && u.Qin;
+    const bool A = (parts & UPD_A) && a.aimg && !a.balance && npb > 0, Q = (parts & UPD_Q) && a.qimg && u.Qin;
     RowExpArgs r{};
     int nz = 0, most = 0;
     auto add = [&](int rows, const double* X, int ld, int* out) {
@@ -1170,22 +1170,24 @@ cudaError_t launch_emu_operands(const EmuUpdArgs& a, bool skip, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_emu_update(const EmuUpdArgs& a, bool operands, cudaStream_t s)
+// V's slices, once for the whole step.
+cudaError_t launch_emu_transforms(const EmuUpdArgs& a, cudaStream_t s)
+{
+    const UpdateArgs& u = a.u;
+    if (!a.vimg || u.npairs <= 0) return cudaSuccess;
+    const int kr = emu_img_rows(u.k);
+    k_emu_vexp<<<dim3((kr + 7) / 8, u.npairs), 256, 0, s>>>(u.V, u.rot, u.k, a.vexp);
+    k_emu_slice_v<<<dim3((u.k + EK - 1) / EK, u.npairs), E_T, 0, s>>>(u.V, u.rot, u.k, a.vexp, a.vimg);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_emu_products(const EmuUpdArgs& a, int parts, cudaStream_t s)
 {
     const UpdateArgs& u = a.u;
     const int nmt = (u.k + EM - 1) / EM, nnt = (u.k + EN - 1) / EN;
-    if (a.vimg && u.npairs > 0) {   // V sliced once for the whole step
-        const int kr = emu_img_rows(u.k);
-        k_emu_vexp<<<dim3((kr + 7) / 8, u.npairs), 256, 0, s>>>(u.V, u.rot, u.k, a.vexp);
-        k_emu_slice_v<<<dim3((u.k + EK - 1) / EK, u.npairs), E_T, 0, s>>>(u.V, u.rot, u.k, a.vexp, a.vimg);
-        cudaError_t e0 = cudaGetLastError();
-        if (e0 != cudaSuccess) return e0;
-        if (operands && (e0 = launch_emu_operands(a, true, s)) != cudaSuccess) return e0;
-        if ((e0 = cudaGetLastError()) != cudaSuccess) return e0;
-    }
     const int npb = u.npairs * (u.npairs - 1) / 2;
-    const int n_sand = npb * nmt * nnt;
-    const int n_q = u.Qin ? u.npairs * ((u.qrows + EM - 1) / EM) * nnt : 0;
+    const int n_sand = parts & UPD_A ? npb * nmt * nnt : 0;
+    const int n_q = (parts & UPD_Q) && u.Qin ? u.npairs * ((u.qrows + EM - 1) / EM) * nnt : 0;
     auto u1 = a.balance ? k_emu_upd1<true> : k_emu_upd1<false>;
     auto u2 = a.balance ? k_emu_upd2<true> : k_emu_upd2<false>;
     cudaError_t e = cudaFuncSetAttribute(u1, cudaFuncAttributeMaxDynamicSharedMemorySize, E_SMEM);

@@ -637,12 +637,12 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_evd(UpdateArgs a, int n_san
 }
 
 template <int MR, int NJ>
-static cudaError_t launch_update_evd_t(const UpdateArgs& a, cudaStream_t s)
+static cudaError_t launch_update_evd_t(const UpdateArgs& a, int parts, cudaStream_t s)
 {
     const int nchunks = (a.k + 8 * NJ - 1) / (8 * NJ);
-    const int n_sand = a.npairs * (a.npairs - 1) / 2 * nchunks;
+    const int n_sand = parts & UPD_A ? a.npairs * (a.npairs - 1) / 2 * nchunks : 0;
     const int H = 32 * MR;
-    const int n_q = a.Qin ? a.npairs * ((a.qrows + H - 1) / H) * nchunks : 0;
+    const int n_q = (parts & UPD_Q) && a.Qin ? a.npairs * ((a.qrows + H - 1) / H) * nchunks : 0;
     const int items = n_sand + n_q;
     if (items == 0) return cudaSuccess;
     const size_t smem = tile_smem_bytes<MR, NJ>(true);
@@ -652,12 +652,25 @@ static cudaError_t launch_update_evd_t(const UpdateArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_update_evd(const UpdateArgs& a, cudaStream_t s)
+cudaError_t launch_update_evd(const UpdateArgs& a, int parts, cudaStream_t s)
 {
-    if (a.k <= 32) return launch_update_evd_t<1, UPD_NJ>(a, s);
-    if (a.k <= 64) return launch_update_evd_t<2, UPD_NJ>(a, s);
-    if (a.k <= 128) return launch_update_evd_t<4, UPD_NJ>(a, s);
-    return launch_update_evd_t<8, UPD_NJ>(a, s);
+    if (a.k <= 32) return launch_update_evd_t<1, UPD_NJ>(a, parts, s);
+    if (a.k <= 64) return launch_update_evd_t<2, UPD_NJ>(a, parts, s);
+    if (a.k <= 128) return launch_update_evd_t<4, UPD_NJ>(a, parts, s);
+    return launch_update_evd_t<8, UPD_NJ>(a, parts, s);
+}
+
+// Nothing for about `ns` nanoseconds, on one thread: holds a side stream back
+// while a kernel of the main one takes its SMs.
+__global__ void k_pause(int ns)
+{
+    for (int i = 0; i < ns; i += 1000) __nanosleep(1000);
+}
+
+cudaError_t launch_pause(int ns, cudaStream_t s)
+{
+    k_pause<<<1, 1, 0, s>>>(ns);
+    return cudaGetLastError();
 }
 
 // ======================================================================== one-sided column update

@@ -872,7 +872,7 @@ PpLaunch pp_launch(int k, int C, bool v32)
 cudaError_t pp_config(const PpLaunch& l, int C, int npairs, cudaLaunchAttribute* attr, cudaLaunchConfig_t* cfg)
 {
     if (!l.kern) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(l.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+    cudaError_t e = cudaFuncSetAttribute(l.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(l.smem, PP_SMEM_MAX));
     if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(l.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     attr->id = cudaLaunchAttributeClusterDimension;
@@ -934,6 +934,9 @@ cudaError_t launch_pivot_pos(const PivotArgs& a, int C, cudaStream_t s)
     const cudaError_t e = pp_config(l, C, a.npairs, attr, &cfg);
     if (e != cudaSuccess) return e;
     cfg.stream = s;
+    // with all of an SM's shared memory no CTA of a kernel that runs beside this
+    // one shares the SM's FP64 unit with the rotation choice
+    if (a.alone) cfg.dynamicSmemBytes = PP_SMEM_MAX;
     return cudaLaunchKernelEx(&cfg, l.kern, a, C);
 }
 

@@ -191,7 +191,7 @@ extern "C" int jacobi_syev_step_noalloc(int np, double* A, int lda, double* Q, i
     ua.V = Vb;
     ua.rot = d_rot;
     ua.cnt = d_cnt;
-    if (launch_update_evd(ua, s) != cudaSuccess) return JACOBI_ERR_CUDA;
+    if (launch_update_evd(ua, UPD_A | UPD_Q, s) != cudaSuccess) return JACOBI_ERR_CUDA;
     if (cudaMemcpy2DAsync(A, (size_t)lda * 8, Anext, bytes, bytes, np, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return JACOBI_ERR_CUDA;
     if (Q && cudaMemcpy2DAsync(Q, (size_t)ldq * 8, Qnext, bytes, bytes, np, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
