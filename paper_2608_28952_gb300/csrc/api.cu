@@ -152,12 +152,12 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
 // Whether the pivot solves leave SMs for a side stream's kernels, and those are
 // worth the events (n = 256: 12.64 ms without, 12.8 with them; n = 500: 33.3 and
 // 31.4).
-static bool sms_left(const EvdState& E)
+static bool sms_left(int np, int npairs, int pcl)
 {
     int dev = 0, sms = 0;
-    return E.np >= 384 && cudaGetDevice(&dev) == cudaSuccess &&
+    return np >= 384 && cudaGetDevice(&dev) == cudaSuccess &&
            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-           E.ord.dev_per_step * E.pcl < sms;
+           npairs * pcl < sms;
 }
 
 // The caller's stream waits for all that the side stream still does.
@@ -181,7 +181,7 @@ SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double
     int sw = sweep0;
     PhaseEvents pe(2 * (size_t)E.ord.S + 1);
     SideStream side;
-    E.side = (E.aimg || E.Qw[0]) && sms_left(E) && side.open() ? &side : nullptr;
+    E.side = (E.aimg || E.Qw[0]) && sms_left(E.np, E.ord.dev_per_step, E.pcl) && side.open() ? &side : nullptr;
     for (; sw < p.max_sweeps; ++sw) {
         const int start = cur;
         auto body = [&](cudaStream_t cs) -> bool {
@@ -393,10 +393,18 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         double* Gw[2] = {ws.get<double>((size_t)m * np), ws.get<double>((size_t)m * np)};
         double* Vw[2] = {vec ? ws.get<double>((size_t)np * np) : nullptr,
                          vec ? ws.get<double>((size_t)np * np) : nullptr};
-        double* Vb = ws.get<double>((size_t)ord.max_pairs * 2 * k * k);
-        int* rot = ws.get<int>(ord.max_pairs);
+        // by step parity: V's update reads one while the next step writes the other
+        const int pcl = choose_pivot_cluster(k, ord.dev_per_step);
+        const bool overlap = vec && sms_left(np, ord.dev_per_step, pcl);
+        double *Vb[2], *part[2];
+        int* rot[2];
+        for (int i = 0; i < 2; ++i) {
+            const bool own = i == 0 || overlap;
+            Vb[i] = own ? ws.get<double>((size_t)ord.max_pairs * 2 * k * k) : Vb[0];
+            rot[i] = own ? ws.get<int>(ord.max_pairs) : rot[0];
+            part[i] = i == 0 || (overlap && emu) ? ws.get<double>((size_t)ord.max_pairs * npanels * k * k) : part[0];
+        }
         double* relmax = ws.get<double>(ord.max_pairs);
-        double* part = ws.get<double>((size_t)ord.max_pairs * npanels * k * k);
         const size_t gsz = pivot_gscratch_doubles(k);
         double* gscr = gsz ? ws.get<double>(gsz * ord.max_pairs) : nullptr;
         int2* dpairs = ws.get<int2>(ord.dev_pairs.size() / 2);
@@ -404,7 +412,6 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         double* norms = ws.get<double>(n);
         int* rank = ws.get<int>(n);
         DevCounters* cnt = ws.get<DevCounters>(1);
-        const int pcl = choose_pivot_cluster(k, ord.dev_per_step);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         int* err = emu ? ws.get<int>(1) : nullptr;
         if (ws.failed) return JACOBI_ERR_ALLOC;
@@ -426,6 +433,8 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         SweepGraph graphs[2];
         bool tried[2] = {false, false}, have[2] = {false, false};
         PhaseEvents pe(3 * (size_t)ord.S + 1);
+        SideStream side;
+        const bool beside = overlap && side.open();
         rc = -1;
         for (sw = 0; sw < p.max_sweeps; ++sw) {
             const int start = cur;
@@ -433,24 +442,36 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                 if (cudaMemsetAsync(sweepmax, 0, sizeof(double), cs) != cudaSuccess) return false;
                 if (cudaEventRecordWithFlags(pe.ev[0], cs, cudaEventRecordExternal) != cudaSuccess) return false;
                 int c = start;
+                // V's update of the last step, owed to the side stream: run beside
+                // the next step's pivot solves (see launch_step)
+                EmuSvdArgs owed_e{};
+                ColUpdateArgs owed{};
+                bool pending = false;
+                auto update_v = [&](int parity) -> bool {
+                    if (!pending) return true;
+                    pending = false;
+                    return (emu ? launch_emu_cols(owed_e, UPD_Q, side.s) : launch_update_cols(owed, UPD_Q, side.s)) == cudaSuccess &&
+                           cudaEventRecord(side.done[parity], side.s) == cudaSuccess;
+                };
                 for (int si = 0; si < ord.S; ++si) {
                     const int nps = ord.dev_per_step, p0 = si * nps;
+                    if (beside && si >= 2 && cudaStreamWaitEvent(cs, side.done[c], 0) != cudaSuccess) return false;
                     EmuSvdArgs sa{Gw[c], Gw[c ^ 1], m, m, Vw[c], Vw[c ^ 1], np, np, dpairs + p0, nps, b, k,
-                                  Vb, rot, part, npanels, prows, err, cnt};
+                                  Vb[c], rot[c], part[c], npanels, prows, err, cnt};
                     if ((emu ? launch_emu_gram(sa, cs)
-                             : launch_gram(Gw[c], m, m, dpairs + p0, nps, b, k, npanels, prows, part, cnt, cs)) != cudaSuccess)
+                             : launch_gram(Gw[c], m, m, dpairs + p0, nps, b, k, npanels, prows, part[c], cnt, cs)) != cudaSuccess)
                         return false;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 1], cs, cudaEventRecordExternal) != cudaSuccess) return false;
                     PivotArgs pa{};
                     pa.ld = np;
-                    pa.gram = part;
+                    pa.gram = part[c];
                     pa.npanels = npanels;
                     pa.pairs = dpairs + p0;
                     pa.npairs = nps;
                     pa.b = b;
                     pa.k = k;
-                    pa.V = Vb;
-                    pa.rot = rot;
+                    pa.V = Vb[c];
+                    pa.rot = rot[c];
                     pa.relmax = relmax;
                     pa.tol_rel = tol;
                     pa.max_sweeps = p.inner_max_sweeps;
@@ -459,7 +480,12 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                     pa.gscratch = gscr;
                     pa.qrws = qrws;
                     pa.cnt = cnt;
+                    pa.alone = beside;
+                    if (beside && cudaEventRecord(side.fork, cs) != cudaSuccess) return false;
                     if (launch_pivot(pa, pcl, cs) != cudaSuccess)
+                        return false;
+                    if (beside && (cudaStreamWaitEvent(side.s, side.fork, 0) != cudaSuccess ||
+                                   (pending && launch_pause(4000, side.s) != cudaSuccess) || !update_v(c ^ 1)))
                         return false;
                     if (launch_max_into(relmax, nps, sweepmax, cs) != cudaSuccess) return false;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 2], cs, cudaEventRecordExternal) != cudaSuccess) return false;
@@ -476,14 +502,21 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                     ca.npairs = nps;
                     ca.b = b;
                     ca.k = k;
-                    ca.Vh = Vb;
-                    ca.rot = rot;
+                    ca.Vh = Vb[c];
+                    ca.rot = rot[c];
                     ca.cnt = cnt;
-                    if ((emu ? launch_emu_cols(sa, cs) : launch_update_cols(ca, cs)) != cudaSuccess) return false;
+                    const int parts = beside ? UPD_A : UPD_A | UPD_Q;
+                    if ((emu ? launch_emu_cols(sa, parts, cs) : launch_update_cols(ca, parts, cs)) != cudaSuccess) return false;
+                    owed_e = sa;
+                    owed = ca;
+                    pending = beside;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 3], cs, cudaEventRecordExternal) != cudaSuccess) return false;
                     c ^= 1;
                 }
-                return true;
+                if (!beside) return true;
+                return cudaEventRecord(side.fork, cs) == cudaSuccess && cudaStreamWaitEvent(side.s, side.fork, 0) == cudaSuccess &&
+                       update_v(c ^ 1) && cudaEventRecord(side.join, side.s) == cudaSuccess &&
+                       cudaStreamWaitEvent(cs, side.join, 0) == cudaSuccess;
             };
             if (!tried[start]) {
                 tried[start] = true;
@@ -837,7 +870,7 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
                                    cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
         SideStream side;
-        E.side = E.aimg && sms_left(E) && side.open() ? &side : nullptr;
+        E.side = E.aimg && sms_left(E.np, E.ord.dev_per_step, E.pcl) && side.open() ? &side : nullptr;
         if (launch_step(E, step, 0, s, p.inner_tol, p.inner_max_sweeps, p.pivot_order) != cudaSuccess ||
             join_side(E, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
@@ -952,7 +985,7 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         ca.Vh = Vb;
         ca.rot = rot;
         ca.cnt = cnt;
-        if ((emu ? launch_emu_cols(sa, s) : launch_update_cols(ca, s)) != cudaSuccess) return JACOBI_ERR_CUDA;
+        if ((emu ? launch_emu_cols(sa, UPD_A | UPD_Q, s) : launch_update_cols(ca, UPD_A | UPD_Q, s)) != cudaSuccess) return JACOBI_ERR_CUDA;
         // columns of pairs outside this step are unchanged: copy them through
         if (cudaMemcpy2DAsync(G, (size_t)ldg * 8, Gw[0], (size_t)m * 8, (size_t)m * 8, np,
                               cudaMemcpyDeviceToDevice, s) != cudaSuccess)

@@ -123,7 +123,7 @@ struct ColUpdateArgs {
     const double* Vh; const int* rot;
     DevCounters* cnt;
 };
-cudaError_t launch_update_cols(const ColUpdateArgs& a, cudaStream_t s);
+cudaError_t launch_update_cols(const ColUpdateArgs& a, int parts, cudaStream_t s);   // parts: UPD_A for G, UPD_Q for V
 
 // Gram partials of one step: for each pair P and row panel r,
 // part[P][r] = G(rows_r, P)^T G(rows_r, P) (k x k).
@@ -261,7 +261,7 @@ struct EmuSvdArgs {
     DevCounters* cnt;
 };
 cudaError_t launch_emu_gram(const EmuSvdArgs& a, cudaStream_t s);
-cudaError_t launch_emu_cols(const EmuSvdArgs& a, cudaStream_t s);
+cudaError_t launch_emu_cols(const EmuSvdArgs& a, int parts, cudaStream_t s);
 size_t emu_update_tbuf_doubles(int npairs, int k);
 cudaError_t launch_offnorm32(int np, const float* Aw, double* partial, unsigned int* ticket,
                              double* result, cudaStream_t s);

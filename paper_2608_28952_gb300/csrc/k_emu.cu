@@ -1211,11 +1211,11 @@ cudaError_t launch_emu_gram(const EmuSvdArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_emu_cols(const EmuSvdArgs& a, cudaStream_t s)
+cudaError_t launch_emu_cols(const EmuSvdArgs& a, int parts, cudaStream_t s)
 {
     const int nnt = (a.k + EN - 1) / EN;
-    const int n_g = a.npairs * ((a.m + EM - 1) / EM) * nnt;
-    const int n_v = a.Vin ? a.npairs * ((a.vrows + EM - 1) / EM) * nnt : 0;
+    const int n_g = !(parts & UPD_A) ? 0 : a.npairs * ((a.m + EM - 1) / EM) * nnt;
+    const int n_v = (parts & UPD_Q) && a.Vin ? a.npairs * ((a.vrows + EM - 1) / EM) * nnt : 0;
     if (n_g + n_v == 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_emu_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, E_SMEM);
     if (e != cudaSuccess) return e;

@@ -731,11 +731,11 @@ __global__ void __launch_bounds__(UPD_T, 2) k_update_cols(ColUpdateArgs a, int n
 }
 
 template <int MR, int NJ>
-static cudaError_t launch_update_cols_t(const ColUpdateArgs& a, cudaStream_t s)
+static cudaError_t launch_update_cols_t(const ColUpdateArgs& a, int parts, cudaStream_t s)
 {
     const int nchunks = (a.k + 8 * NJ - 1) / (8 * NJ), H = 32 * MR;
-    const int n_g = a.npairs * ((a.m + H - 1) / H) * nchunks;
-    const int n_v = a.Vin ? a.npairs * ((a.vrows + H - 1) / H) * nchunks : 0;
+    const int n_g = parts & UPD_A ? a.npairs * ((a.m + H - 1) / H) * nchunks : 0;
+    const int n_v = (parts & UPD_Q) && a.Vin ? a.npairs * ((a.vrows + H - 1) / H) * nchunks : 0;
     if (n_g + n_v == 0) return cudaSuccess;
     const size_t smem = tile_smem_bytes<MR, NJ>(false);
     cudaError_t e = cudaFuncSetAttribute(k_update_cols<MR, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -745,10 +745,10 @@ static cudaError_t launch_update_cols_t(const ColUpdateArgs& a, cudaStream_t s)
 }
 
 // Tiles of 128 rows (fewer loads of Vhat) while they fill the GPU, else of 32.
-cudaError_t launch_update_cols(const ColUpdateArgs& a, cudaStream_t s)
+cudaError_t launch_update_cols(const ColUpdateArgs& a, int parts, cudaStream_t s)
 {
     const int tiles = a.npairs * ((a.m + 127) / 128 + (a.Vin ? (a.vrows + 127) / 128 : 0)) * ((a.k + 7) / 8);
-    return tiles >= 8 * UPD_SMS ? launch_update_cols_t<4, UPD_NJ>(a, s) : launch_update_cols_t<1, UPD_NJ>(a, s);
+    return tiles >= 8 * UPD_SMS ? launch_update_cols_t<4, UPD_NJ>(a, parts, s) : launch_update_cols_t<1, UPD_NJ>(a, parts, s);
 }
 
 // ======================================================================== Gram (split K over rows)
