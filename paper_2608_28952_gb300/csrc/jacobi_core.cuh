@@ -230,7 +230,15 @@ __device__ __forceinline__ int schur2_sign(double d, double apq)
     return (__double_as_longlong(d) << 1) == 0 ? 0 : (__double2hiint(d) ^ __double2hiint(apq)) & 0x80000000;
 }
 
+// The batched forms' choice: the seeds of schur2_wide, whose rounding their
+// results (the signs of eigenvectors among them) have always had.
 __device__ __forceinline__ void schur2(double app, double aqq, double apq, double& s, double& t, double& tau)
+{
+    schur2_wide(rn_sub(aqq, app), apq, s, t, tau);
+}
+
+// The pivot solves' choice (k_pivot_pos splits it over two lanes).
+__device__ __forceinline__ void schur2_pivot(double app, double aqq, double apq, double& s, double& t, double& tau)
 {
     const double d = rn_sub(aqq, app);
     const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(apq);

@@ -1052,7 +1052,7 @@ __global__ void k_rotation_params(int count, const double* __restrict__ app, con
     double* o = out + (size_t)8 * i;
     double s = 0.0, t = 0.0, tau = 0.0;
     const bool on = rotation_wanted(p, q, x, tol);
-    if (x != 0.0) schur2(p, q, x, s, t, tau);
+    if (x != 0.0) schur2_pivot(p, q, x, s, t, tau);
     o[0] = t;
     o[1] = s;
     o[2] = tau;

@@ -1,4 +1,4 @@
-// k_pivot_pos.cu -- the pivot solves of one step, C in {1, 2, 4, 8} CTAs per
+// k_pivot_pos.cu -- the pivot solves of one step, C = 1 .. 16 CTAs per
 // pair (a thread-block cluster when C > 1): Algorithm 2 applied with b = 1 to
 // each 2b x 2b pivot in the round-robin order, the diagonal carried as
 // hi + lo.
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // where the FP64 unit bounds the round, not where the rotation choice does
     // and would wait behind four more FP64 warps (one quad per bulk thread;
     // measured: k = 32 78 us with V after the quads, 82 us beside them; k = 128
-    // with 16 pairs 613 and 520)
+    // with 16 pairs 613 and 520 us)
     constexpr bool kAuxV = V32 || (AT > 0 && QPT > 1);
     // and carry the diagonal, unless an FP64 V keeps them busy (then the first
     // bulk threads do, and the chain reads its part of the diagonal itself)
