@@ -54,8 +54,10 @@ cudaMemPool_t pool_here()
     }();
     int dev = -1;
     unsigned long long id = 0;
-    if (!ctx_id || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices || cudaFree(nullptr) != cudaSuccess ||
-        ctx_id(nullptr, &id) != CUDA_SUCCESS) {
+    // (a thread without a context gets the device's primary one; cudaFree(nullptr)
+    // would do that too, but is refused while any thread captures a graph)
+    if (!ctx_id || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices ||
+        (ctx_id(nullptr, &id) != CUDA_SUCCESS && (cudaSetDevice(dev) != cudaSuccess || ctx_id(nullptr, &id) != CUDA_SUCCESS))) {
         cudaGetLastError();
         return nullptr;
     }
