@@ -216,6 +216,7 @@ struct Fork {
     int used = 0;
     bool ok = true;
     Fork(jacobi_plan* p, cudaStream_t st) : pl(p), s(st) {}
+    ~Fork() { join(); }   // also where a launch failed: the caller's stream waits for what was launched
     // a side stream (made when first wanted, kept by the plan); s when there is none left
     cudaStream_t next()
     {
@@ -236,6 +237,7 @@ struct Fork {
         for (int i = 0; i < used; ++i)
             ok = cudaEventRecord(pl->ev_join[i], pl->side[i]) == cudaSuccess &&
                  cudaStreamWaitEvent(s, pl->ev_join[i], 0) == cudaSuccess && ok;
+        used = 0;
         return ok ? cudaSuccess : cudaErrorUnknown;
     }
 };
