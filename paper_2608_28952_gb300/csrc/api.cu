@@ -149,17 +149,6 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
     return e;
 }
 
-// Whether the pivot solves leave SMs for a side stream's kernels, and those are
-// worth the events (n = 256: 12.64 ms without, 12.8 with them; n = 500: 33.3 and
-// 31.4).
-static bool sms_left(int np, int npairs, int pcl)
-{
-    int dev = 0, sms = 0;
-    return np >= 384 && cudaGetDevice(&dev) == cudaSuccess &&
-           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-           npairs * pcl < sms;
-}
-
 // The caller's stream waits for all that the side stream still does.
 static cudaError_t join_side(EvdState& E, cudaStream_t cs)
 {
@@ -181,7 +170,7 @@ SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double
     int sw = sweep0;
     PhaseEvents pe(2 * (size_t)E.ord.S + 1);
     SideStream side;
-    E.side = (E.aimg || E.Qw[0]) && sms_left(E.np, E.ord.dev_per_step, E.pcl) && side.open() ? &side : nullptr;
+    E.side = E.Vb[1] != E.Vb[0] && side.open() ? &side : nullptr;
     for (; sw < p.max_sweeps; ++sw) {
         const int start = cur;
         auto body = [&](cudaStream_t cs) -> bool {
@@ -259,10 +248,8 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
         E.Aw[1] = ws.get<double>(np2);
         E.Qw[0] = vec ? ws.get<double>(np2) : nullptr;
         E.Qw[1] = vec ? ws.get<double>(np2) : nullptr;
-        for (int i = 0; i < 2; ++i) {
-            E.Vb[i] = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
-            E.rot[i] = ws.get<int>(E.ord.max_pairs);
-        }
+        E.Vb[0] = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
+        E.rot[0] = ws.get<int>(E.ord.max_pairs);
         const size_t gsz = pivot_gscratch_doubles(E.k);
         E.gscratch = gsz ? ws.get<double>(gsz * E.ord.max_pairs) : nullptr;
         E.dpairs = ws.get<int2>(E.ord.dev_pairs.size() / 2);
@@ -277,10 +264,8 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
             E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, E.k));
             E.err = ws.get<int>(1);
             if (emu_image_wanted()) {
-                for (int i = 0; i < 2; ++i) {
-                    E.vimg[i] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
-                    E.vexp[i] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
-                }
+                E.vimg[0] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
+                E.vexp[0] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
                 if (p.conv != JACOBI_CONV_REL) {   // (balanced products slice per tile)
                     E.aimg = ws.get<unsigned char>(emu_update_aimg_bytes(E.ord.dev_per_step, E.k));
                     E.atab = ws.get<int>((size_t)E.ord.dev_per_step * E.np);
@@ -292,6 +277,7 @@ static int syev_fp64(int n, double* A, int lda, double* w, double* Q, int ldq,
             }
         }
         E.balance = p.conv == JACOBI_CONV_REL;
+        E.parity_buffers(ws);
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (E.err && cudaMemsetAsync(E.err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(E.dpairs, E.ord.dev_pairs.data(), E.ord.dev_pairs.size() * sizeof(int),
@@ -373,6 +359,22 @@ extern "C" int jacobi_syev(int n, double* A, int lda, double* w, double* Q, int 
     return rc;
 }
 
+// The Gram partials of a step, the last thing a call cannot do without: of
+// small panels where those suit the step and fit, else of 512 rows.
+static double* gram_partials(Workspace& ws, int m, int npairs, int max_pairs, int k, bool emu, int* prows, int* npanels)
+{
+    *prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, npairs, k);
+    for (;;) {
+        *npanels = (m + *prows - 1) / *prows;
+        double* p = ws.try_get<double>((size_t)max_pairs * *npanels * k * k);
+        if (p) return p;
+        if (*prows >= gram_panel_rows()) break;
+        *prows = gram_panel_rows();
+    }
+    ws.failed = true;
+    return nullptr;
+}
+
 // ============================================================================ SVD (FP64)
 static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V, int ldv,
                       const jacobi_params& p, jacobi_stats* st, cudaStream_t s)
@@ -385,25 +387,15 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
     const bool vec = p.want_vectors != 0;
     const double tol = std::max(p.tol, sqrt((double)m) * U64);
     const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
-    const int prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, ord.dev_per_step, k);
-    const int npanels = (m + prows - 1) / prows;
     int rc = 0;
     {
         Workspace ws(s);
         double* Gw[2] = {ws.get<double>((size_t)m * np), ws.get<double>((size_t)m * np)};
         double* Vw[2] = {vec ? ws.get<double>((size_t)np * np) : nullptr,
                          vec ? ws.get<double>((size_t)np * np) : nullptr};
-        // by step parity: V's update reads one while the next step writes the other
         const int pcl = choose_pivot_cluster(k, ord.dev_per_step);
-        const bool overlap = vec && sms_left(np, ord.dev_per_step, pcl);
-        double *Vb[2], *part[2];
-        int* rot[2];
-        for (int i = 0; i < 2; ++i) {
-            const bool own = i == 0 || overlap;
-            Vb[i] = own ? ws.get<double>((size_t)ord.max_pairs * 2 * k * k) : Vb[0];
-            rot[i] = own ? ws.get<int>(ord.max_pairs) : rot[0];
-            part[i] = i == 0 || (overlap && emu) ? ws.get<double>((size_t)ord.max_pairs * npanels * k * k) : part[0];
-        }
+        double* Vb[2] = {ws.get<double>((size_t)ord.max_pairs * 2 * k * k)};
+        int* rot[2] = {ws.get<int>(ord.max_pairs)};
         double* relmax = ws.get<double>(ord.max_pairs);
         const size_t gsz = pivot_gscratch_doubles(k);
         double* gscr = gsz ? ws.get<double>(gsz * ord.max_pairs) : nullptr;
@@ -414,6 +406,25 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         DevCounters* cnt = ws.get<DevCounters>(1);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         int* err = emu ? ws.get<int>(1) : nullptr;
+        int prows, npanels;
+        double* part[2] = {gram_partials(ws, m, ord.dev_per_step, ord.max_pairs, k, emu, &prows, &npanels)};
+        // by step parity, where they fit: V's update reads one while the next step
+        // writes the other
+        Vb[1] = Vb[0];
+        rot[1] = rot[0];
+        part[1] = part[0];
+        bool overlap = false;
+        if (!ws.failed && vec && sms_left(np, ord.dev_per_step, pcl)) {
+            double* v = ws.try_get<double>((size_t)ord.max_pairs * 2 * k * k);
+            int* r = v ? ws.try_get<int>(ord.max_pairs) : nullptr;
+            double* g = r && emu ? ws.try_get<double>((size_t)ord.max_pairs * npanels * k * k) : part[0];
+            if (r && g) {
+                overlap = true;
+                Vb[1] = v;
+                rot[1] = r;
+                part[1] = g;
+            }
+        }
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),
                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -825,10 +836,8 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
         E.Aw[1] = ws.get<double>(np2);
         E.Qw[0] = Q ? ws.get<double>(np2) : nullptr;
         E.Qw[1] = Q ? ws.get<double>(np2) : nullptr;
-        for (int i = 0; i < 1; ++i) {
-            E.Vb[i] = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
-            E.rot[i] = ws.get<int>(E.ord.max_pairs);
-        }
+        E.Vb[0] = ws.get<double>((size_t)E.ord.max_pairs * 2 * E.k * E.k);
+        E.rot[0] = ws.get<int>(E.ord.max_pairs);
         const size_t gsz = pivot_gscratch_doubles(E.k);
         E.gscratch = gsz ? ws.get<double>(gsz * E.ord.max_pairs) : nullptr;
         E.dpairs = ws.get<int2>(E.ord.dev_pairs.size() / 2);
@@ -839,10 +848,8 @@ extern "C" int jacobi_syev_step(int np, double* A, int lda, double* Q, int ldq,
             E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, E.k));
             E.err = ws.get<int>(1);
             if (emu_image_wanted()) {
-                for (int i = 0; i < 1; ++i) {
-                    E.vimg[i] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
-                    E.vexp[i] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
-                }
+                E.vimg[0] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, E.k));
+                E.vexp[0] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, E.k));
                 if (p.conv != JACOBI_CONV_REL) {   // (balanced products slice per tile)
                     E.aimg = ws.get<unsigned char>(emu_update_aimg_bytes(E.ord.dev_per_step, E.k));
                     E.atab = ws.get<int>((size_t)E.ord.dev_per_step * E.np);
@@ -912,8 +919,6 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
     const double tol = std::max(p.tol, sqrt((double)m) * U64);
     const int nps = ord.dev_per_step, p0 = step * nps;
     const bool emu = p.precision == JACOBI_PREC_FP64_EMU || p.fp64_products == 1;
-    const int prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, nps, k);
-    const int npanels = (m + prows - 1) / prows;
     {
         Workspace ws(s);
         double* Gw[2] = {ws.get<double>((size_t)m * np), ws.get<double>((size_t)m * np)};
@@ -922,7 +927,6 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         double* Vb = ws.get<double>((size_t)ord.max_pairs * 2 * k * k);
         int* rot = ws.get<int>(ord.max_pairs);
         double* relmax = ws.get<double>(ord.max_pairs);
-        double* part = ws.get<double>((size_t)ord.max_pairs * npanels * k * k);
         const size_t gsz = pivot_gscratch_doubles(k);
         double* gscr = gsz ? ws.get<double>(gsz * ord.max_pairs) : nullptr;
         int2* dpairs = ws.get<int2>(ord.dev_pairs.size() / 2);
@@ -931,6 +935,8 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         const int pcl = choose_pivot_cluster(k, nps);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         int* err = emu ? ws.get<int>(1) : nullptr;
+        int prows, npanels;
+        double* part = gram_partials(ws, m, nps, ord.max_pairs, k, emu, &prows, &npanels);
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (err && cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),

@@ -209,10 +209,8 @@ int syev_mixed(int n, double* A, int lda, double* w, double* Q, int ldq, const j
     E.Qw[1] = ws.get<double>(np2);
     double* A0p = ws.get<double>(np2);
     double* lam = ws.get<double>(np);
-    for (int i = 0; i < 2; ++i) {
-        E.Vb[i] = ws.get<double>((size_t)E.ord.max_pairs * 2 * k * k);
-        E.rot[i] = ws.get<int>(E.ord.max_pairs);
-    }
+    E.Vb[0] = ws.get<double>((size_t)E.ord.max_pairs * 2 * k * k);
+    E.rot[0] = ws.get<int>(E.ord.max_pairs);
     const size_t gsz = pivot_gscratch_doubles(k);
     E.gscratch = gsz ? ws.get<double>(gsz * E.ord.max_pairs) : nullptr;
     E.dpairs = ws.get<int2>(E.ord.dev_pairs.size() / 2);
@@ -239,10 +237,8 @@ int syev_mixed(int n, double* A, int lda, double* w, double* Q, int ldq, const j
         E.T64 = ws.get<double>(emu_update_tbuf_doubles(E.ord.dev_per_step, k));
         E.err = L.err;
         if (emu_image_wanted()) {
-            for (int i = 0; i < 2; ++i) {
-                E.vimg[i] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, k));
-                E.vexp[i] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, k));
-            }
+            E.vimg[0] = ws.get<unsigned char>(emu_update_vimg_bytes(E.ord.dev_per_step, k));
+            E.vexp[0] = ws.get<int>(emu_update_vexp_ints(E.ord.dev_per_step, k));
             if (p.conv != JACOBI_CONV_REL) {   // (balanced products slice per tile)
                 E.aimg = ws.get<unsigned char>(emu_update_aimg_bytes(E.ord.dev_per_step, k));
                 E.atab = ws.get<int>((size_t)E.ord.dev_per_step * np);
@@ -257,6 +253,7 @@ int syev_mixed(int n, double* A, int lda, double* w, double* Q, int ldq, const j
             gimg[1] = ws.get<unsigned char>(emu_gemm_img_bytes(np, np));
         }
     }
+    E.parity_buffers(ws);
     if (ws.failed) return JACOBI_ERR_ALLOC;
     L.pcl = E.pcl;
     L.dpairs = E.dpairs;

@@ -32,15 +32,19 @@ struct Workspace {
     template <class T>
     T* get(size_t count)
     {
-        if (count == 0) count = 1;
-        const size_t bytes = count * sizeof(T);
-        if (failed || bytes > limit - used) {
-            failed = true;
-            return nullptr;
-        }
+        T* p = try_get<T>(count);
+        if (!p) failed = true;
+        return p;
+    }
+    // For what a call can do without: null where it does not fit (asked for
+    // after everything the call needs).
+    template <class T>
+    T* try_get(size_t count)
+    {
+        const size_t bytes = (count == 0 ? 1 : count) * sizeof(T);
+        if (failed || bytes > limit - used) return nullptr;
         void* p = nullptr;
         if (workspace_alloc(&p, bytes, s) != cudaSuccess) {
-            failed = true;
             cudaGetLastError();
             return nullptr;
         }
@@ -193,6 +197,17 @@ inline int choose_pivot_cluster(int k, int npairs)
     return pivot_cluster_size(k, npairs, (size_t)smem);
 }
 
+// Whether the pivot solves leave SMs for a side stream's kernels, and those are
+// worth the events (n = 256: 12.64 ms without, 12.8 with them; n = 500: 33.3 and
+// 31.4).
+inline bool sms_left(int np, int npairs, int pcl)
+{
+    int dev = 0, sms = 0;
+    return np >= 384 && cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           npairs * pcl < sms;
+}
+
 inline int check_params(const jacobi_params& p)
 {
     if (p.b < 1) return -7;
@@ -255,6 +270,26 @@ struct EvdState {
     bool pending = false;         // Q's update of the last step is still to be launched there
     EmuUpdArgs pending_q{};
     int pending_cur = 0;
+
+    // The odd steps' transforms: buffers of their own where a side stream may
+    // read the even steps' meanwhile and they fit, else the even steps'.
+    void parity_buffers(Workspace& ws)
+    {
+        Vb[1] = Vb[0];
+        rot[1] = rot[0];
+        vimg[1] = vimg[0];
+        vexp[1] = vexp[0];
+        if (ws.failed || !(aimg || Qw[0]) || !sms_left(np, ord.dev_per_step, pcl)) return;
+        double* v = ws.try_get<double>((size_t)ord.max_pairs * 2 * k * k);
+        int* r = v ? ws.try_get<int>(ord.max_pairs) : nullptr;
+        unsigned char* vi = r && vimg[0] ? ws.try_get<unsigned char>(emu_update_vimg_bytes(ord.dev_per_step, k)) : nullptr;
+        int* ve = vi ? ws.try_get<int>(emu_update_vexp_ints(ord.dev_per_step, k)) : nullptr;
+        if (!r || (vimg[0] && !ve)) return;
+        Vb[1] = v;
+        rot[1] = r;
+        vimg[1] = vi;
+        vexp[1] = ve;
+    }
     // pivot_order == 2: the per-pair QRCP scratch of the pivoting step
     double* qrws = nullptr;
     // emulated products: balance by the diagonal (relative stop criterion)
