@@ -91,8 +91,7 @@ __device__ __forceinline__ bool rotation_wanted(T app, T aqq, T apq, T tol)
 // rotation) in place of about 40 with single FP32 seeds, two FP64 Newton steps
 // and hardware conversions.  t is within 2u of the exact root, tau and s within
 // 4u, (1 - s tau)^2 + s^2 = 1 within 2u (measured over 2e7 triples): the rotation
-// applied in Rutishauser's or the three-shear form stays orthogonal to working
-// precision.
+// applied in Rutishauser's form stays orthogonal to working precision.
 __device__ __forceinline__ int f64_biased_exp(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
 __device__ __forceinline__ float rsqrt_seed(float x)

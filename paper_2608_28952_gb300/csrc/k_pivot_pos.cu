@@ -120,17 +120,25 @@ __device__ __forceinline__ void pp_st2(uint32_t a, double x, double y)
 __device__ __forceinline__ void pp_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void pp_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-// (x, y) <- (c x - s y, s x + c y) as three shears with tau = s / (1 + c):
-// x1 = x - tau y, y' = y + s x1, x' = x1 - tau y'.  Three FMAs where the
-// two-correction form x - s (y + tau x), y + s (x - tau y) takes four; each
-// shear is exactly invertible, so the pair is orthogonal as far as s and tau
-// belong together, and every rounding is relative to the entry it makes.
-template <typename T>
-__device__ __forceinline__ void shear2(T s, T tau, T& x, T& y)
+// The rotation of a quad.  Rutishauser's form (rot2: four FMAs for two entries)
+// rounds each entry once at full size.  Three shears, x1 = x - tau y, y' = y + s x1,
+// x' = x1 - tau y', take three FMAs but round x twice: V's loss of orthogonality
+// over a solve is 1.25 times rot2's and the errors of singular values and
+// residuals 1.15 to 1.25 times (measured, svd 300 x 60 to 2000 x 300).  So an FP64
+// result takes rot2 throughout; the shears rotate the FP64 quads of the
+// low-precision sweeps alone, which leave as FP32 (the same error against 64 bits
+// to two digits, n = 8192, b = 128: one step 4.43 ms, 4.95 with rot2 there; FP64
+// solves pay 1.5 % for theirs at n = 64 to 1000, svd 1000 x 200 5 %).
+template <bool V32>
+__device__ __forceinline__ void quad_rot(double s, double tau, double& x, double& y)
 {
-    const T u = fma(-tau, y, x);
-    y = fma(s, u, y);
-    x = fma(-tau, y, u);
+    if constexpr (V32) {
+        const double u = fma(-tau, y, x);
+        y = fma(s, u, y);
+        x = fma(-tau, y, u);
+    } else {
+        rot2(s, tau, x, y);
+    }
 }
 
 __device__ __forceinline__ double f64_flip(double x, int sign_bit)   // no FP64 instruction
@@ -421,7 +429,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
 #pragma unroll
                 for (int u = 0; u < U; ++u)
                     if (on[u]) {
-                        shear2(ps[u], pu[u], xt[u], xb[u]);
+                        rot2(ps[u], pu[u], xt[u], xb[u]);
                         Vl[ot[u] + o] = xt[u];
                         Vl[ob[u] + o] = xb[u];
                     }
@@ -539,10 +547,10 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
             for (int u = 0; u < QPT; ++u) {
                 if (tid + u * NB < nq) {
                     const double2 pi = par[so + (ij[u] & 0xff)], pj = par[so + (ij[u] >> 8)];
-                    shear2(pi.x, pi.y, x[u][0], x[u][2]);
-                    shear2(pi.x, pi.y, x[u][1], x[u][3]);
-                    shear2(pj.x, pj.y, x[u][0], x[u][1]);
-                    shear2(pj.x, pj.y, x[u][2], x[u][3]);
+                    quad_rot<V32>(pi.x, pi.y, x[u][0], x[u][2]);
+                    quad_rot<V32>(pi.x, pi.y, x[u][1], x[u][3]);
+                    quad_rot<V32>(pj.x, pj.y, x[u][0], x[u][1]);
+                    quad_rot<V32>(pj.x, pj.y, x[u][2], x[u][3]);
                 }
             }
             may_store();
