@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // and would wait behind four more FP64 warps (one quad per bulk thread;
     // measured: k = 32 78 us with V after the quads, 82 us beside them; k = 128
     // with 16 pairs 613 and 520 us)
-    constexpr bool kAuxV = V32 || (AT > 0 && QPT > 1);
+    constexpr bool kAuxV = AT > 0 && (V32 || QPT > 1);
     // and carry the diagonal, unless an FP64 V keeps them busy (then the first
     // bulk threads do, and the chain reads its part of the diagonal itself)
     constexpr bool kAuxDiag = AT >= CH && (V32 || !kAuxV);
@@ -388,8 +388,8 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     const int ve0 = vwarp ? vt >> 5 : vt / rows, vi0 = vwarp ? vt & 31 : vt - ve0 * rows;
     const int vde = vwarp ? VN / 32 : VN / rows, vdi = vwarp ? 0 : VN - vde * rows;
     auto rotate_v = [&](int so, int rd) {
-        constexpr int U = NB == 256 && !V32 ? 2 : 4;   // items in flight: 4 (256 bulk threads: 2 of each row group,
-        constexpr int UO = NB == 256 && !V32 ? 4 : 1;  // which costs fewer registers)
+        constexpr int U = NB > 128 && !kAuxV ? 2 : 4;   // items in flight: 4 (256 bulk threads and more: 2 of each row
+        constexpr int UO = NB > 128 && !kAuxV ? 4 : 1;  // group, which costs fewer registers)
         int e = ve0, i = vi0;
         while (e < h) {
             int ot[U], ob[U];
@@ -830,17 +830,25 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
 using PpKernel = void (*)(PivotArgs, int);
 
 // 128 bulk threads while they hold a CTA's quads in registers (four warps fill
-// the FP64 unit), else 256.  A block's warps per SM quarter set the registers
-// a thread may use: with 128 bulk threads, 4 auxiliary warps fit; with 256 the
-// diagonal goes to bulk threads and an FP32 V to one warp.
+// the FP64 unit), else 256, or 288 for the few largest shares that shared
+// memory still takes (2b = 184 and 186 with C = 2, 224 with 3; one step of 76 pairs,
+// b = 92, low precision: 8.8 ms, 14.8 with one CTA per pair).  A block's warps
+// per SM quarter set the registers a thread may use: with 128 bulk threads, 4
+// auxiliary warps fit; with 256 the diagonal goes to bulk threads and an FP32 V
+// to one warp, with 288 both go to bulk threads.  Null where no instance holds
+// the share.
 template <bool V32>
 PpKernel pp_kernel(int chunk, int chain, int& nb, int& at)
 {
-    nb = chunk > 128 * PP_QMAX ? 256 : 128;
+    nb = chunk > 256 * PP_QMAX ? 288 : (chunk > 128 * PP_QMAX ? 256 : 128);
     const int qpt = (chunk + nb - 1) / nb;
+    if (nb == 288) {
+        at = 0;
+        return qpt <= PP_QMAX && chain <= 96 ? k_pivot_pos<288, PP_QMAX, 96, 0, V32> : nullptr;
+    }
     if (nb == 256) {
         at = V32 ? 32 : 0;
-        if (qpt > PP_QMAX) return nullptr;
+        if (chain > 128) return nullptr;
         return chain <= 96 ? k_pivot_pos<256, PP_QMAX, 96, V32 ? 32 : 0, V32> : k_pivot_pos<256, PP_QMAX, 128, V32 ? 32 : 0, V32>;
     }
     at = 128;
@@ -899,7 +907,8 @@ cudaError_t pp_config(const PpLaunch& l, int C, int npairs, cudaLaunchAttribute*
 
 bool pivot_pos_fits(int k, int C, size_t smem_cap)
 {
-    return C <= PP_MAXC && (C == 1 || k / C >= 8) && pp_smem(k, C, false).bytes + PP_STATIC <= smem_cap;
+    return C <= PP_MAXC && (C == 1 || k / C >= 8) && pp_smem(k, C, false).bytes + PP_STATIC <= smem_cap &&
+           pp_launch(k, C, false).kern && pp_launch(k, C, true).kern;
 }
 
 // Cluster size for a step with npairs pairs: the largest C whose
