@@ -359,20 +359,27 @@ extern "C" int jacobi_syev(int n, double* A, int lda, double* w, double* Q, int 
     return rc;
 }
 
-// The Gram partials of a step, the last thing a call cannot do without: of
-// small panels where those suit the step and fit, else of 512 rows.
-static double* gram_partials(Workspace& ws, int m, int npairs, int max_pairs, int k, bool emu, int* prows, int* npanels)
+// The Gram partials of a step, the last thing a call cannot do without: one for
+// each panel where those fit, else one for all of a pair's panels (FP64 panels
+// of less than 512 rows only: what they need beyond 512-row ones is the step's
+// choice).  The sums are the same, bit for bit (gram_panel_rows_for).
+struct GramPartials {
+    double* p = nullptr;
+    int rows, prows, npanels;   // rows of a panel, of a partial; partials
+};
+static GramPartials gram_partials(Workspace& ws, int m, int npairs, int max_pairs, int k, bool emu)
 {
-    *prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, npairs, k);
-    for (;;) {
-        *npanels = (m + *prows - 1) / *prows;
-        double* p = ws.try_get<double>((size_t)max_pairs * *npanels * k * k);
-        if (p) return p;
-        if (*prows >= gram_panel_rows()) break;
-        *prows = gram_panel_rows();
+    GramPartials g;
+    g.rows = g.prows = emu ? gram_panel_rows() : gram_panel_rows_for(m, npairs, k);
+    g.npanels = (m + g.rows - 1) / g.rows;
+    g.p = ws.try_get<double>((size_t)max_pairs * g.npanels * k * k);
+    if (!g.p && g.rows < gram_panel_rows()) {
+        g.npanels = 1;
+        g.prows = m;
+        g.p = ws.try_get<double>((size_t)max_pairs * k * k);
     }
-    ws.failed = true;
-    return nullptr;
+    if (!g.p) ws.failed = true;
+    return g;
 }
 
 // ============================================================================ SVD (FP64)
@@ -406,8 +413,8 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         DevCounters* cnt = ws.get<DevCounters>(1);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         int* err = emu ? ws.get<int>(1) : nullptr;
-        int prows, npanels;
-        double* part[2] = {gram_partials(ws, m, ord.dev_per_step, ord.max_pairs, k, emu, &prows, &npanels)};
+        const GramPartials gp = gram_partials(ws, m, ord.dev_per_step, ord.max_pairs, k, emu);
+        double* part[2] = {gp.p};
         // by step parity, where they fit: V's update reads one while the next step
         // writes the other
         Vb[1] = Vb[0];
@@ -417,7 +424,7 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         if (!ws.failed && vec && sms_left(np, ord.dev_per_step, pcl)) {
             double* v = ws.try_get<double>((size_t)ord.max_pairs * 2 * k * k);
             int* r = v ? ws.try_get<int>(ord.max_pairs) : nullptr;
-            double* g = r && emu ? ws.try_get<double>((size_t)ord.max_pairs * npanels * k * k) : part[0];
+            double* g = r && emu ? ws.try_get<double>((size_t)ord.max_pairs * gp.npanels * k * k) : part[0];
             if (r && g) {
                 overlap = true;
                 Vb[1] = v;
@@ -468,15 +475,15 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                     const int nps = ord.dev_per_step, p0 = si * nps;
                     if (beside && si >= 2 && cudaStreamWaitEvent(cs, side.done[c], 0) != cudaSuccess) return false;
                     EmuSvdArgs sa{Gw[c], Gw[c ^ 1], m, m, Vw[c], Vw[c ^ 1], np, np, dpairs + p0, nps, b, k,
-                                  Vb[c], rot[c], part[c], npanels, prows, err, cnt};
+                                  Vb[c], rot[c], part[c], gp.npanels, gp.prows, err, cnt};
                     if ((emu ? launch_emu_gram(sa, cs)
-                             : launch_gram(Gw[c], m, m, dpairs + p0, nps, b, k, npanels, prows, part[c], cnt, cs)) != cudaSuccess)
+                             : launch_gram(Gw[c], m, m, dpairs + p0, nps, b, k, gp.npanels, gp.prows, gp.rows, part[c], cnt, cs)) != cudaSuccess)
                         return false;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 1], cs, cudaEventRecordExternal) != cudaSuccess) return false;
                     PivotArgs pa{};
                     pa.ld = np;
                     pa.gram = part[c];
-                    pa.npanels = npanels;
+                    pa.npanels = gp.npanels;
                     pa.pairs = dpairs + p0;
                     pa.npairs = nps;
                     pa.b = b;
@@ -935,8 +942,8 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
         const int pcl = choose_pivot_cluster(k, nps);
         double* qrws = p.pivot_order == 2 ? ws.get<double>((size_t)ord.max_pairs * b * k) : nullptr;
         int* err = emu ? ws.get<int>(1) : nullptr;
-        int prows, npanels;
-        double* part = gram_partials(ws, m, nps, ord.max_pairs, k, emu, &prows, &npanels);
+        const GramPartials gp = gram_partials(ws, m, nps, ord.max_pairs, k, emu);
+        double* part = gp.p;
         if (ws.failed) return JACOBI_ERR_ALLOC;
         if (err && cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return JACOBI_ERR_CUDA;
         if (cudaMemcpyAsync(dpairs, ord.dev_pairs.data(), ord.dev_pairs.size() * sizeof(int),
@@ -950,14 +957,14 @@ extern "C" int jacobi_gesvd_step(int m, int np, double* G, int ldg, double* V, i
                                    cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             return JACOBI_ERR_CUDA;
         EmuSvdArgs sa{Gw[0], Gw[1], m, m, Vw[0], Vw[1], np, np, dpairs + p0, nps, b, k,
-                      Vb, rot, part, npanels, prows, err, cnt};
-        if ((emu ? launch_emu_gram(sa, s) : launch_gram(Gw[0], m, m, dpairs + p0, nps, b, k, npanels, prows, part, cnt, s)) !=
+                      Vb, rot, part, gp.npanels, gp.prows, err, cnt};
+        if ((emu ? launch_emu_gram(sa, s) : launch_gram(Gw[0], m, m, dpairs + p0, nps, b, k, gp.npanels, gp.prows, gp.rows, part, cnt, s)) !=
             cudaSuccess)
             return JACOBI_ERR_CUDA;
         PivotArgs pa{};
         pa.ld = np;
         pa.gram = part;
-        pa.npanels = npanels;
+        pa.npanels = gp.npanels;
         pa.pairs = dpairs + p0;
         pa.npairs = nps;
         pa.b = b;

@@ -126,11 +126,12 @@ struct ColUpdateArgs {
 cudaError_t launch_update_cols(const ColUpdateArgs& a, int parts, cudaStream_t s);   // parts: UPD_A for G, UPD_Q for V
 
 // Gram partials of one step: for each pair P and row panel r,
-// part[P][r] = G(rows_r, P)^T G(rows_r, P) (k x k).
+// part[P][r] = G(rows_r, P)^T G(rows_r, P) (k x k), prows rows each, summed over
+// panels of `rows` rows (prows: that, or all rows).
 int gram_panel_rows();                               // emulated products
 int gram_panel_rows_for(int m, int npairs, int k);   // FP64
 cudaError_t launch_gram(const double* G, int ldg, int m, const int2* pairs, int npairs, int b, int k, int npanels,
-                        int prows, double* part, DevCounters* cnt, cudaStream_t s);
+                        int prows, int rows, double* part, DevCounters* cnt, cudaStream_t s);
 
 // Finalisation (EVD): w <- sorted diag(Aw)[0:n] (ascending, stable), Q(:, j)
 // <- Qw(0:n, perm j), A <- Aw(0:n, 0:n).

@@ -757,7 +757,10 @@ int gram_panel_rows() { return GRAM_ROWS; }
 // Rows of a panel for the FP64 Gram blocks: 512 (few partials to sum) while the
 // panels fill the GPU, else as few as 64 (a 512-row panel of a 32 x 32 block is
 // 126 us of one SM; 7 pairs of 1000 rows were 14 such items: 1000 x 200, b = 16,
-// Gram and update 202 -> 41 us per step).
+// Gram and update 202 -> 41 us per step).  The panels fix the sum: each panel's
+// rows in order, then the panels in order.  An item takes prows rows: one panel,
+// or (where the partials of all panels don't fit) all of them, which it adds in
+// that order: the same bits.
 int gram_panel_rows_for(int m, int npairs, int k)
 {
     int rows = GRAM_ROWS;
@@ -765,13 +768,13 @@ int gram_panel_rows_for(int m, int npairs, int k)
     return rows;
 }
 
-// Item (pair e, panel r, column chunk c): rows c0.. of the k x k Gram block
-// (lower triangle only: rows >= c0), K = the panel's rows of G.
-template <int MR, int NJ>
+// Item (pair e, partial r, column chunk c; ALL: of all panels): rows c0.. of the k x k Gram block
+// (lower triangle only: rows >= c0), K = the partial's rows of G.
+template <int MR, int NJ, bool ALL>
 __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G, int ldg, int m,
                                                   const int2* __restrict__ pairs, int b, int k,
-                                                  int npanels, int prows, int nchunks, double* __restrict__ part,
-                                                  DevCounters* cnt)
+                                                  int npanels, int prows, int rows, int nchunks,
+                                                  double* __restrict__ part, DevCounters* cnt)
 {
     extern __shared__ __align__(16) double sm[];
     constexpr int AS_LD = 32 * MR + 1, TN = 8 * NJ, T_LD = TN + 1;
@@ -788,20 +791,27 @@ __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G,
     const int row0 = c0;  // lower triangle: output rows >= first column of the chunk
     const int M = k - row0, mr = (M + 31) >> 5;
     const int g0 = pr * prows, K = min(prows, m - g0);
-    Tile<MR, NJ> t;
-    t.zero();
-    gemm_tile<MR, NJ, true, false, true>(
-        t, M, K, mr,
-        [&](int mm, int kk) { return G[(g0 + kk) + (size_t)ldg * pair_map(I, J, b, row0 + mm)]; },
-        [&](int kk, int j) { return j < kw ? G[(g0 + kk) + (size_t)ldg * pair_map(I, J, b, c0 + j)] : 0.0; },
-        As, Bs, nullptr);
+    Tile<MR, NJ> t, sum;
+    for (int p0 = g0; p0 < g0 + K; p0 += rows) {
+        t.zero();
+        gemm_tile<MR, NJ, true, false, true>(
+            t, M, min(rows, g0 + K - p0), mr,
+            [&](int mm, int kk) { return G[(p0 + kk) + (size_t)ldg * pair_map(I, J, b, row0 + mm)]; },
+            [&](int kk, int j) { return j < kw ? G[(p0 + kk) + (size_t)ldg * pair_map(I, J, b, c0 + j)] : 0.0; },
+            As, Bs, nullptr);
+        if constexpr (!ALL) break;
+#pragma unroll
+        for (int i = 0; i < MR; ++i)
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) sum.acc[i][j] = p0 == g0 ? t.acc[i][j] : sum.acc[i][j] + t.acc[i][j];
+    }
     double* out = part + ((size_t)e * npanels + pr) * k * k;
 #pragma unroll
     for (int i = 0; i < MR; ++i)
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             const int mm = ty + 32 * i, jj = tx + 8 * j;
-            if (i < mr && mm < M && jj < kw) out[(row0 + mm) + (size_t)k * (c0 + jj)] = t.acc[i][j];
+            if (i < mr && mm < M && jj < kw) out[(row0 + mm) + (size_t)k * (c0 + jj)] = ALL ? sum.acc[i][j] : t.acc[i][j];
         }
     if (tid == 0) {
         atomicAdd(&cnt->flops_fp64, 2ull * M * K * kw);
@@ -811,21 +821,22 @@ __global__ void __launch_bounds__(UPD_T, 2) k_gram(const double* __restrict__ G,
 
 template <int MR, int NJ>
 static cudaError_t launch_gram_t(const double* G, int ldg, int m, const int2* pairs, int npairs, int b, int k, int npanels,
-                                 int prows, double* part, DevCounters* cnt, cudaStream_t s)
+                                 int prows, int rows, double* part, DevCounters* cnt, cudaStream_t s)
 {
     const int nchunks = (k + 8 * NJ - 1) / (8 * NJ);
     const size_t smem = tile_smem_bytes<MR, NJ>(false);
-    cudaError_t e = cudaFuncSetAttribute(k_gram<MR, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = prows > rows ? k_gram<MR, NJ, true> : k_gram<MR, NJ, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_gram<MR, NJ><<<npairs * npanels * nchunks, UPD_T, smem, s>>>(G, ldg, m, pairs, b, k, npanels, prows, nchunks, part, cnt);
+    kern<<<npairs * npanels * nchunks, UPD_T, smem, s>>>(G, ldg, m, pairs, b, k, npanels, prows, rows, nchunks, part, cnt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gram(const double* G, int ldg, int m, const int2* pairs, int npairs, int b, int k, int npanels, int prows,
-                        double* part, DevCounters* cnt, cudaStream_t s)
+                        int rows, double* part, DevCounters* cnt, cudaStream_t s)
 {
     if (npairs * npanels == 0) return cudaSuccess;
-    auto go = [&](auto f) { return f(G, ldg, m, pairs, npairs, b, k, npanels, prows, part, cnt, s); };
+    auto go = [&](auto f) { return f(G, ldg, m, pairs, npairs, b, k, npanels, prows, rows, part, cnt, s); };
     if (k <= 32) return go(launch_gram_t<1, UPD_NJ>);
     if (k <= 64) return go(launch_gram_t<2, UPD_NJ>);
     if (k <= 128) return go(launch_gram_t<4, UPD_NJ>);
