@@ -260,12 +260,14 @@ __device__ __forceinline__ void schur2_pivot(double app, double aqq, double apq,
 // 2^-18 of 1 needs FP64.  There, where every operand lies in [2^-400, 2^400],
 // the squares can neither overflow nor underflow and nonnegative doubles
 // compare like their bit patterns; elsewhere the square-root form.
-// The FP32 part: 1 rotate, 0 skip, -1 undecided; y = the leading parts of tol
-// tol app aqq multiplied, esum = the sum of their biased exponents.
+// The FP32 part: 1 rotate, 0 skip, -1 undecided (subnormals, infinities and NaN
+// too: they have no leading bits to compare); y = the leading parts of tol tol app
+// aqq multiplied, esum = the sum of their biased exponents.
+__device__ __forceinline__ bool f64_normal_exp(int e) { return (unsigned)(e - 1) < 2046u; }
 __device__ __forceinline__ int rotation_wanted_lead(double apq, float y, int esum)
 {
     const int ep = f64_biased_exp(apq), sh = esum - 2 * ep - 2046;   // rhs / lhs in [2^(sh - 2), 2^(sh + 4))
-    if (ep < 1) return (__double_as_longlong(apq) << 1) == 0 ? 0 : -1;
+    if (!f64_normal_exp(ep)) return (__double_as_longlong(apq) << 1) == 0 ? 0 : -1;
     const float fa = f64_lead(apq), x = fa * fa, r = y * __int_as_float((min(max(sh, -9), 9) + 127) << 23);
     if (sh > 8) return 0;
     if (sh < -8) return 1;
@@ -285,7 +287,7 @@ __device__ __forceinline__ bool rotation_wanted(double app, double aqq, double a
 {
     if ((__double_as_longlong(apq) << 1) == 0) return false;
     const int e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq), et = f64_biased_exp(tol);
-    if (e1 >= 1 && e2 >= 1 && et >= 1) {
+    if (f64_normal_exp(e1) && f64_normal_exp(e2) && f64_normal_exp(et)) {
         const float ft = f64_lead(tol);
         const int w = rotation_wanted_lead(apq, (ft * ft) * (f64_lead(app) * f64_lead(aqq)), e1 + e2 + 2 * et);
         if (w >= 0) return w;

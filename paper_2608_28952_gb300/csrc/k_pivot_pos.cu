@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // leading parts of a pair's diagonal for the next choice
     auto prepare = [&](double app, double aqq, double d) {
         const int e1 = f64_biased_exp(app), e2 = f64_biased_exp(aqq);
-        const bool ok = e1 >= 1 && e2 >= 1 && tol_e >= 1;
+        const bool ok = f64_normal_exp(e1) && f64_normal_exp(e2) && f64_normal_exp(tol_e);
         return make_float4(f64_lead(d), f64_rest(d), tol_f * (f64_lead(app) * f64_lead(aqq)),
                            __int_as_float(ok ? e1 + e2 + 2 * tol_e : -1));
     };
