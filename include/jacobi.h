@@ -442,7 +442,8 @@ int jacobi_syev_step_noalloc(int np, double* A, int lda, double* Q, int ldq,
  * Algorithm 1 applied with b = 1), for `count` triples (app[i], aqq[i],
  * apq[i]) in device memory.  For each i, out[8 i .. 8 i + 7] (device) gets
  * t, s, tau and the rotation test (1.0 rotate, 0.0 skip) as the pivot solves
- * compute them (FP32 seeds refined by Newton steps in FP64), then t, s, tau
+ * compute them (seeds in pairs of FP32 numbers, one Newton step in FP64; the
+ * batched FP64 solves refine single FP32 seeds by two), then t, s, tau
  * and the test by the textbook formulas in correctly rounded FP64 operations
  * (zeta = (aqq - app)/(2 apq), t = sgn(zeta)/(|zeta| + sqrt(1 + zeta^2)),
  * c = 1/sqrt(1 + t^2), s = t c, tau = s/(1 + c); rotate when

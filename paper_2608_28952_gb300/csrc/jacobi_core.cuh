@@ -131,10 +131,6 @@ __device__ __forceinline__ float f32_of(double x)
     const long long m = (v >> 29) - (896ll << 23);
     return m < 0x00800000 ? 0.0f : __int_as_float((int)m | (__double2hiint(x) & 0x80000000));
 }
-__device__ __forceinline__ double f64_signed(double x, int sign_bit)
-{
-    return __hiloint2double(__double2hiint(x) | sign_bit, __double2loint(x));
-}
 
 // any finite triple, by FP32 seeds and FP64 Newton steps on scaled values
 __device__ __forceinline__ void schur2_wide(double d, double apq, double& s, double& t, double& tau)
@@ -236,22 +232,48 @@ __device__ __forceinline__ void schur2(double app, double aqq, double apq, doubl
     schur2_wide(rn_sub(aqq, app), apq, s, t, tau);
 }
 
-// The pivot solves' choice (k_pivot_pos splits it over two lanes).
+// The pivot solves' choice in the two halves that two lanes share there.  A half: t
+// and z = tau or c, all for |d| and |apq| (dh, dl: d's leading parts); false
+// where the pairs of floats don't serve.
+__device__ __forceinline__ bool schur2_half(double d, double apq, float dh, float dl, bool want_c, double& t, double& z)
+{
+    const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(apq);
+    if (!schur2_paired(Ed, Ea)) return false;
+    float t0, te;
+    t = schur2_t(fabs(apq), Ea, fabs(d), Ed, dh, dl, t0, te);
+    z = schur2_z(t, t0, te, want_c);
+    return true;
+}
+__device__ __forceinline__ double f64_flip(double x, int sign_bit)   // no FP64 instruction
+{
+    return __hiloint2double(__double2hiint(x) ^ sign_bit, __double2loint(x));
+}
+// The halves joined (t, tau and c as both left them): signs, s, and every triple
+// that the pairs of floats don't take.  flip: zeta = 0 picks t = -1 (the pair's
+// indices are in descending order).
+__device__ __forceinline__ void schur2_join(double d, double apq, bool paired, bool flip, double& s, double& t, double& tau, double& c)
+{
+    int sgn = schur2_sign(d, apq);
+    s = t * c;
+    if (!paired) {
+        schur2_wide(d, apq, s, t, tau);
+        c = fma(-s, tau, 1.0);
+        sgn = 0;
+    }
+    if (flip && (__double_as_longlong(d) << 1) == 0) sgn = 0x80000000;
+    s = f64_flip(s, sgn);
+    t = f64_flip(t, sgn);
+    tau = f64_flip(tau, sgn);
+}
+// The same by one thread.
 __device__ __forceinline__ void schur2_pivot(double app, double aqq, double apq, double& s, double& t, double& tau)
 {
     const double d = rn_sub(aqq, app);
-    const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(apq);
-    if (!schur2_paired(Ed, Ea)) {
-        schur2_wide(d, apq, s, t, tau);
-        return;
-    }
-    const int sgn = schur2_sign(d, apq);
-    float t0, te;
-    const double ta = schur2_t(fabs(apq), Ea, fabs(d), Ed, f64_lead(d), f64_rest(d), t0, te);
-    const double ca = schur2_z(ta, t0, te, true);
-    t = f64_signed(ta, sgn);
-    tau = f64_signed(schur2_z(ta, t0, te, false), sgn);
-    s = f64_signed(ta * ca, sgn);
+    const float dh = f64_lead(d), dl = f64_rest(d);
+    double c = 1.0;
+    const bool paired = schur2_half(d, apq, dh, dl, false, t, tau);
+    schur2_half(d, apq, dh, dl, true, t, c);
+    schur2_join(d, apq, paired, false, s, t, tau, c);
 }
 
 // |apq| > tol sqrt|app| sqrt|aqq| as apq^2 > tol^2 |app| |aqq|, first on
@@ -339,14 +361,6 @@ struct CoreSmem {
 template <typename T> struct Pair2;
 template <> struct Pair2<float> { using type = float2; };
 template <> struct Pair2<double> { using type = double2; };
-
-// Quad (e1, e2), e1 < e2 < half, of flat index qi = e2 (e2 - 1) / 2 + e1.
-__device__ __forceinline__ void quad_of(const unsigned* qtab, int qi, int& e1, int& e2)
-{
-    const unsigned qq = qtab[qi];
-    e1 = qq & 0xffff;
-    e2 = qq >> 16;
-}
 
 // Solve the packed symmetric k x k matrix Ap (k even) in place by blockDim.x
 // threads.  V (k x k, column-major, ld k) accumulates the rotations when not

@@ -141,11 +141,6 @@ __device__ __forceinline__ void quad_rot(double s, double tau, double& x, double
     }
 }
 
-__device__ __forceinline__ double f64_flip(double x, int sign_bit)   // no FP64 instruction
-{
-    return __hiloint2double(__double2hiint(x) ^ sign_bit, __double2loint(x));
-}
-
 template <bool V32> struct PpV { using T = double; };
 template <> struct PpV<true> { using T = float; };
 
@@ -606,28 +601,12 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
             int want = es >= 0 ? rotation_wanted_lead(av, f.z, es) : -1;
             if (want < 0) want = (__double_as_longlong(av) << 1) != 0 && rotation_wanted_exact(ad.x, ad.y, av, tol);
             const bool on = mine && want;
-            const int Ed = f64_biased_exp(d), Ea = f64_biased_exp(av);
-            const bool paired = schur2_paired(Ed, Ea);
-            double t = 0.0, z = 0.0;
-            float t0 = 0.0f, te = 0.0f;
-            if (on && paired) {
-                t = schur2_t(fabs(av), Ea, fabs(d), Ed, f.x, f.y, t0, te);
-                z = schur2_z(t, t0, te, lead);
-            }
+            double s, t = 0.0, z = 0.0;
+            const bool paired = on && schur2_half(d, av, f.x, f.y, lead, t, z);
             const double zo = __shfl_xor_sync(0xffffffffu, z, 1);
-            double tau = lead ? zo : z, c = lead ? z : zo, s = t * c;
-            if (on) {
-                int sgn = schur2_sign(d, av);
-                if (!paired) {
-                    schur2_wide(d, av, s, t, tau);
-                    c = fma(-s, tau, 1.0);
-                    sgn = 0;
-                }
-                // zeta = 0: t = +1 with the smaller index as p
-                if ((__double_as_longlong(d) << 1) == 0 && pp_index(ce, rd, nr) > pp_index(k - 1 - ce, rd, nr)) sgn = 0x80000000;
-                s = f64_flip(s, sgn);
-                t = f64_flip(t, sgn);
-                tau = f64_flip(tau, sgn);
+            double tau = lead ? zo : z, c = lead ? z : zo;
+            if (on) {   // zeta = 0: t = +1 with the smaller index as p
+                schur2_join(d, av, paired, pp_index(ce, rd, nr) > pp_index(k - 1 - ce, rd, nr), s, t, tau, c);
             } else {
                 s = t = tau = 0.0;
                 c = 1.0;

@@ -54,6 +54,14 @@ extern "C" void wanted(int n, const double* p, const double* q, const double* x,
 {
     for (int i = 0; i < n; ++i) out[i] = jac::rotation_wanted(p[i], q[i], x[i], tol);
 }
+extern "C" void params(int n, const double* p, const double* q, const double* x, int pivot, double off, double* t, double* s, double* tau)
+{
+    g_off = off;
+    for (int i = 0; i < n; ++i)
+        if (pivot) jac::schur2_pivot(p[i], q[i], x[i], s[i], t[i], tau[i]);
+        else jac::schur2(p[i], q[i], x[i], s[i], t[i], tau[i]);
+}
+extern "C" int paired(double d, double x) { return jac::schur2_paired(jac::f64_biased_exp(d), jac::f64_biased_exp(x)); }
 """
 
 
@@ -94,3 +102,44 @@ def test_rotation_test_on_special_values(core, tol):
         near = np.abs(np.abs(x) - rhs) <= 1e-12 * rhs     # (the form without square roots rounds elsewhere)
     bad = (out != want) & ~(near & np.isfinite(rhs))
     assert not bad.any(), list(zip(p[bad], q[bad], x[bad], out[bad]))[:8]
+
+
+def _triples(seed):
+    """Magnitudes 1e-280 to 1e280; within a triple close together, or up to 1e20 and
+    1e60 apart; equal and negative diagonals."""
+    r = np.random.default_rng(seed)
+    n = 40000
+    base = 10.0 ** r.uniform(-280, 280, n)
+    p, q = (base * r.standard_normal(n) * 10.0 ** r.uniform(-3, 3, n) for _ in range(2))
+    x = base * r.standard_normal(n) * 10.0 ** r.choice([0.0, -5.0, -12.0, -17.0, -20.0, -60.0, 4.0], n)
+    q[: n // 8] = p[: n // 8]
+    p[n // 8: n // 4] *= -1
+    ok = (np.abs(x) > 1e-290) & np.isfinite(p) & np.isfinite(q)
+    return [np.ascontiguousarray(a[ok]) for a in (p, q, x)]
+
+
+@pytest.mark.parametrize("off", [0.0, 2.0 ** -22, -2.0 ** -22])
+@pytest.mark.parametrize("pivot", [1, 0])
+def test_rotation_parameters(core, pivot, off):
+    """t, s and tau of the pivot solves' choice (the halves that two lanes share,
+    joined) and of the batched solves', with the seeds off by their bound, against
+    the textbook formulas in long double: within 6 units of 2^-53, and (1 - s tau)^2 +
+    s^2 = 1 within 8, the bounds that the kernels' results are held to."""
+    p, q, x = _triples(11 + pivot)
+    t, s, tau = (np.zeros(p.size) for _ in range(3))
+    core.params(p.size, _p(p), _p(q), _p(x), pivot, C.c_double(off), _p(t), _p(s), _p(tau))
+    d = q - p
+    if pivot:      # both kinds of triple are among them
+        kind = {core.paired(C.c_double(a), C.c_double(b)) for a, b in zip(d[:4000], x[:4000])}
+        assert kind == {0, 1}
+    L = np.longdouble
+    with np.errstate(all="ignore"):
+        zeta = L(d) / (L(2) * L(x))
+        tt = np.where(zeta >= 0, L(1), L(-1)) / (np.abs(zeta) + np.sqrt(L(1) + zeta * zeta))
+    cc = L(1) / np.sqrt(L(1) + tt * tt)
+    for name, got, want in (("t", t, tt), ("s", s, tt * cc), ("tau", tau, tt * cc / (L(1) + cc))):
+        err = np.abs((L(got) - want) / want).astype(np.float64)
+        err = err[np.abs(want) > 1e-290]
+        assert err.max() <= 6 * U, (name, err.max() / U)
+    c = 1.0 - s * tau
+    assert np.abs(c * c + s * s - 1.0).max() <= 8 * U
