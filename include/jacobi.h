@@ -16,7 +16,7 @@
  *     (host pointers) or the argument is named h_*;
  *   - the caller owns every buffer; the library allocates its workspace
  *     stream-ordered on the given stream and frees it before returning, from
- *     a memory pool of its own per device that holds on to at most 8 GiB
+ *     a memory pool of its own per context that holds on to at most 8 GiB
  *     between calls (the driver takes it back when an allocation of the
  *     process would otherwise fail);
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default

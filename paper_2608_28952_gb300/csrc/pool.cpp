@@ -5,7 +5,7 @@
 // system at the call's last synchronisation, and the next call mapped it anew:
 // about 2.7 ms for each GB (GB300: 11 of the 22 ms of one emulated FP64 step at
 // n = 8192, 4 of the 7.5 ms of a low-precision one).  The library keeps one
-// pool of its own per device that holds on to at most kPoolKeep bytes between
+// pool of its own per context that holds on to at most kPoolKeep bytes between
 // calls.  The driver takes unused bytes back from it when any allocation of the
 // process would otherwise fail (measured: cudaMalloc of 3 GB more than was
 // free, with 6.4 GB held, succeeds and leaves the pool empty), and a call that
@@ -13,8 +13,9 @@
 //
 // The pool is the driver's: it is safe with several threads, and memory freed
 // on one stream and reused on another is ordered by the driver.  A pool
-// belongs to a context; after cudaDeviceReset the old handle is dropped (the
-// context's id tells) and a new pool made.
+// belongs to a context and goes with it: each context has its own, found by the
+// context's id, which no later context gets (after cudaDeviceReset a device has
+// a new one).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -27,7 +28,7 @@ namespace jac {
 namespace {
 
 constexpr unsigned long long kPoolKeep = 8ull << 30;   // 3 % of the device's memory
-constexpr int kPoolDevices = 64;
+constexpr int kPoolContexts = 64;   // looked after at once; beyond them the first one's entry is used anew
 
 struct Entry {
     unsigned long long ctx = 0;
@@ -35,7 +36,8 @@ struct Entry {
 };
 
 std::mutex g_mu;
-Entry g_pool[kPoolDevices];
+Entry g_pool[kPoolContexts];
+int g_next = 0;
 
 using CtxGetId = CUresult (*)(CUcontext, unsigned long long*);
 
@@ -56,15 +58,14 @@ cudaMemPool_t pool_here()
     unsigned long long id = 0;
     // (a thread without a context gets the device's primary one; cudaFree(nullptr)
     // would do that too, but is refused while any thread captures a graph)
-    if (!ctx_id || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices ||
+    if (!ctx_id || cudaGetDevice(&dev) != cudaSuccess ||
         (ctx_id(nullptr, &id) != CUDA_SUCCESS && (cudaSetDevice(dev) != cudaSuccess || ctx_id(nullptr, &id) != CUDA_SUCCESS))) {
         cudaGetLastError();
         return nullptr;
     }
     std::lock_guard<std::mutex> lock(g_mu);
-    Entry& e = g_pool[dev];
-    if (e.pool && e.ctx == id) return e.pool;
-    e = Entry{};
+    for (const Entry& e : g_pool)
+        if (e.pool && e.ctx == id) return e.pool;
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -80,8 +81,8 @@ cudaMemPool_t pool_here()
         cudaMemPoolDestroy(p);
         return nullptr;
     }
-    e.ctx = id;
-    e.pool = p;
+    g_pool[g_next] = Entry{id, p};
+    g_next = (g_next + 1) % kPoolContexts;
     return p;
 }
 
