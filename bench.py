@@ -769,8 +769,8 @@ def run_gpu(args, wl):
         # Gram (lower triangle, split-K) + column update of G and V, per step
         alg = P * (m_eff * k * k + 2 * m_eff * k * k + 2 * npd * k * k)
         if kc["launches"]:
-            # the update class counts two launches per step (Gram, columns)
-            per = kc["launches"] // 2 if dom == "update" else kc["launches"]
+            # the update class has two or three launches per step (Gram, columns of G and of V); a step one pivot launch
+            per = kernels["pivot"]["launches"] if dom == "update" else kc["launches"]
             avg_ms, per_launch = kc["ms"] / max(per, 1), kc["flops"] / max(per, 1)
         else:
             avg_ms, per_launch = kc["ms"], kc["flops"]

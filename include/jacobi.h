@@ -174,10 +174,17 @@ typedef struct {
     double ms_total;         /* device time of the call (CUDA events)          */
     double ms_pivot;         /* device time in the pivot-solve kernels         */
     double ms_update;        /* device time in the update kernels (A and Q /
-                                G and V; for the SVD including the Gram)        */
-    long long launches;      /* kernels this call launched                     */
+                                G and V; for the SVD including the Gram).  Q's
+                                and V's updates may run beside the pivot solves
+                                on a stream of their own: they count here all
+                                the same, so the two can add up to more than
+                                ms_total                                       */
+    long long launches;      /* kernels this call launched (the kernels of one
+                                emulated update count as one)                  */
     long long pivot_launches;  /* of which pivot-solve kernels                 */
-    long long update_launches; /* of which update kernels                      */
+    long long update_launches; /* of which update kernels (A and Q, or G and V,
+                                together, or one each where Q's or V's runs
+                                beside the pivot solves)                       */
     double flops_fp64;       /* FP64 flops issued (updates + pivot solves; a
                                 V accumulated in FP32 is not counted)          */
     double flops_update;     /* of which in the update / Gram kernels          */

@@ -133,15 +133,22 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
     if ((e = launch_pivot(pa, E.pcl, cs)) != cudaSuccess) return e;
     if (mid && (e = cudaEventRecordWithFlags(mid, cs, cudaEventRecordExternal)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(sd.s, sd.fork, 0)) != cudaSuccess) return e;
-    if (E.T64 && ((e = launch_emu_operands(ea, UPD_A, false, sd.s)) != cudaSuccess ||
-                  (e = cudaEventRecord(sd.join, sd.s)) != cudaSuccess))
+    SideTimes* tm = E.times;
+    const size_t t0 = 2 * (size_t)first;
+    if (E.T64 && ((tm && (e = tm->open(t0, sd.s)) != cudaSuccess) ||
+                  (e = launch_emu_operands(ea, UPD_A, false, sd.s)) != cudaSuccess ||
+                  (e = cudaEventRecord(sd.join, sd.s)) != cudaSuccess ||
+                  (tm && (e = tm->close(t0, sd.s)) != cudaSuccess)))
         return e;
     if (E.pending && (e = launch_pause(4000, sd.s)) != cudaSuccess) return e;
+    const bool timed = tm && (E.pending || E.T64);
+    if (timed && (e = tm->open(t0 + 1, sd.s)) != cudaSuccess) return e;
     if ((e = update_q_pending(E)) != cudaSuccess) return e;
     if (E.T64 && ((e = launch_emu_operands(ea, UPD_Q, false, sd.s)) != cudaSuccess ||
                   (e = launch_emu_transforms(ea, cs)) != cudaSuccess ||
                   (e = cudaStreamWaitEvent(cs, sd.join, 0)) != cudaSuccess))
         return e;
+    if (timed && (e = tm->close(t0 + 1, sd.s)) != cudaSuccess) return e;
     e = E.T64 ? launch_emu_products(ea, UPD_A, cs) : launch_update_evd(ua, UPD_A, cs);
     E.pending = ua.Qin != nullptr;
     E.pending_q = ea;
@@ -154,8 +161,11 @@ static cudaError_t join_side(EvdState& E, cudaStream_t cs)
 {
     if (!E.side) return cudaSuccess;
     cudaError_t e;
+    const bool timed = E.times && E.pending;
+    const size_t last = 2 * (size_t)E.ord.S;
     if ((e = cudaEventRecord(E.side->fork, cs)) != cudaSuccess || (e = cudaStreamWaitEvent(E.side->s, E.side->fork, 0)) != cudaSuccess ||
-        (e = update_q_pending(E)) != cudaSuccess || (e = cudaEventRecord(E.side->join, E.side->s)) != cudaSuccess)
+        (timed && (e = E.times->open(last, E.side->s)) != cudaSuccess) || (e = update_q_pending(E)) != cudaSuccess ||
+        (timed && (e = E.times->close(last, E.side->s)) != cudaSuccess) || (e = cudaEventRecord(E.side->join, E.side->s)) != cudaSuccess)
         return e;
     return cudaStreamWaitEvent(cs, E.side->join, 0);
 }
@@ -171,6 +181,8 @@ SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double
     PhaseEvents pe(2 * (size_t)E.ord.S + 1);
     SideStream side;
     E.side = E.Vb[1] != E.Vb[0] && side.open() ? &side : nullptr;
+    SideTimes times(E.side ? 2 * (size_t)E.ord.S + 1 : 0);
+    E.times = E.side ? &times : nullptr;
     for (; sw < p.max_sweeps; ++sw) {
         const int start = cur;
         auto body = [&](cudaStream_t cs) -> bool {
@@ -205,9 +217,12 @@ SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double
             st->ms_pivot += pe.ms(2 * si, 2 * si + 1);
             st->ms_update += pe.ms(2 * si + 1, 2 * si + 2);
         }
-        st->launches += 2 * E.ord.S + 1;
+        st->ms_update += times.ms();
+        // on a side stream Q's updates are launches of their own, with a pause before all but the last
+        const int q_own = E.side && E.Qw[0] ? E.ord.S : 0;
+        st->launches += 2 * E.ord.S + 1 + (q_own ? 2 * q_own - 1 : 0);
         st->pivot_launches += E.ord.S;
-        st->update_launches += E.ord.S;
+        st->update_launches += E.ord.S + q_own;
         const double off = sqrt(h_res[0]);
         const double meas = use_rel ? h_res[2] : off;
         if (sw < 64) {
@@ -453,6 +468,7 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
         PhaseEvents pe(3 * (size_t)ord.S + 1);
         SideStream side;
         const bool beside = overlap && side.open();
+        SideTimes times(beside ? (size_t)ord.S : 0);   // V's updates
         rc = -1;
         for (sw = 0; sw < p.max_sweeps; ++sw) {
             const int start = cur;
@@ -465,11 +481,12 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                 EmuSvdArgs owed_e{};
                 ColUpdateArgs owed{};
                 bool pending = false;
-                auto update_v = [&](int parity) -> bool {
+                auto update_v = [&](int parity, int step) -> bool {
                     if (!pending) return true;
                     pending = false;
-                    return (emu ? launch_emu_cols(owed_e, UPD_Q, side.s) : launch_update_cols(owed, UPD_Q, side.s)) == cudaSuccess &&
-                           cudaEventRecord(side.done[parity], side.s) == cudaSuccess;
+                    return times.open(step, side.s) == cudaSuccess &&
+                           (emu ? launch_emu_cols(owed_e, UPD_Q, side.s) : launch_update_cols(owed, UPD_Q, side.s)) == cudaSuccess &&
+                           cudaEventRecord(side.done[parity], side.s) == cudaSuccess && times.close(step, side.s) == cudaSuccess;
                 };
                 for (int si = 0; si < ord.S; ++si) {
                     const int nps = ord.dev_per_step, p0 = si * nps;
@@ -503,7 +520,7 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                     if (launch_pivot(pa, pcl, cs) != cudaSuccess)
                         return false;
                     if (beside && (cudaStreamWaitEvent(side.s, side.fork, 0) != cudaSuccess ||
-                                   (pending && launch_pause(4000, side.s) != cudaSuccess) || !update_v(c ^ 1)))
+                                   (pending && launch_pause(4000, side.s) != cudaSuccess) || !update_v(c ^ 1, si - 1)))
                         return false;
                     if (launch_max_into(relmax, nps, sweepmax, cs) != cudaSuccess) return false;
                     if (cudaEventRecordWithFlags(pe.ev[3 * si + 2], cs, cudaEventRecordExternal) != cudaSuccess) return false;
@@ -533,7 +550,7 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                 }
                 if (!beside) return true;
                 return cudaEventRecord(side.fork, cs) == cudaSuccess && cudaStreamWaitEvent(side.s, side.fork, 0) == cudaSuccess &&
-                       update_v(c ^ 1) && cudaEventRecord(side.join, side.s) == cudaSuccess &&
+                       update_v(c ^ 1, ord.S - 1) && cudaEventRecord(side.join, side.s) == cudaSuccess &&
                        cudaStreamWaitEvent(cs, side.join, 0) == cudaSuccess;
             };
             if (!tried[start]) {
@@ -556,9 +573,11 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                 st->ms_update += pe.ms(3 * si, 3 * si + 1) + pe.ms(3 * si + 2, 3 * si + 3);
                 st->ms_pivot += pe.ms(3 * si + 1, 3 * si + 2);
             }
-            st->launches += 4 * ord.S;
+            st->ms_update += times.ms();
+            // on a side stream V's updates are launches of their own, with a pause before all but the last
+            st->launches += 4 * ord.S + (beside ? 2 * ord.S - 1 : 0);
             st->pivot_launches += ord.S;
-            st->update_launches += 2 * ord.S;
+            st->update_launches += 2 * ord.S + (beside ? ord.S : 0);
             if (sw < 64) st->off_hist[sw] = mx;
             if (sw == 0) st->off_initial = mx;
             st->off_final = mx;

@@ -107,6 +107,27 @@ struct PhaseEvents {
     }
 };
 
+// Intervals on a side stream (its update kernels), by number; those that a sweep
+// did not open count nothing.
+struct SideTimes {
+    PhaseEvents pe;
+    std::vector<char> on;
+    explicit SideTimes(size_t n) : pe(2 * n), on(n, 0) {}
+    cudaError_t open(size_t i, cudaStream_t s)
+    {
+        on[i] = 1;
+        return cudaEventRecordWithFlags(pe.ev[2 * i], s, cudaEventRecordExternal);
+    }
+    cudaError_t close(size_t i, cudaStream_t s) { return cudaEventRecordWithFlags(pe.ev[2 * i + 1], s, cudaEventRecordExternal); }
+    double ms() const
+    {
+        double t = 0.0;
+        for (size_t i = 0; i < on.size(); ++i)
+            if (on[i]) t += pe.ms(2 * i, 2 * i + 1);
+        return t;
+    }
+};
+
 // A low-priority stream beside the caller's, with the events that fork from it
 // and join it again.  Destroyed only after its work is done.
 struct SideStream {
@@ -270,6 +291,7 @@ struct EvdState {
     bool pending = false;         // Q's update of the last step is still to be launched there
     EmuUpdArgs pending_q{};
     int pending_cur = 0;
+    SideTimes* times = nullptr;   // two intervals a step (the images of A's operands; Q's) and the last step's Q
 
     // The odd steps' transforms: buffers of their own where a side stream may
     // read the even steps' meanwhile and they fit, else the even steps'.
