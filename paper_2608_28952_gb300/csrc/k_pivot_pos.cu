@@ -117,6 +117,7 @@ __device__ __forceinline__ void pp_st2(uint32_t a, double x, double y)
 {
     asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(x), "d"(y) : "memory");
 }
+__device__ __forceinline__ void pp_block_barrier(int threads) { asm volatile("barrier.sync 2, %0;" ::"r"(threads) : "memory"); }
 __device__ __forceinline__ void pp_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void pp_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
@@ -225,9 +226,11 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     int* s_ce = s_own + h;                                // this CTA's chain pairs
     __shared__ int s_nce, s_cntg[4], s_nr, s_r1;
     __shared__ double s_red[(NB + CH + AT) / 32], s_part[PP_MAXC];
+    // (the roles run rounds of their own, so they meet at a barrier with a thread
+    // count: a __syncthreads() has to be one and the same for the whole block)
     auto sync_all = [&] {
         if (C == 1) {
-            __syncthreads();
+            pp_block_barrier(nt);
         } else {
             pp_arrive();
             pp_wait();
@@ -236,7 +239,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // "every quad of the round is in registers": only with one buffer
     auto loaded = [&] {
         if (L.two) return;
-        if (C == 1) __syncthreads();
+        if (C == 1) pp_block_barrier(nt);
         else pp_arrive();
     };
     auto may_store = [&] {
@@ -486,7 +489,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                 pr_f[de] = prepare(dv, other, df);
                 pr_d[de] = df;
             }
-            asm volatile("bar.arrive 1, %0;" ::"r"(pair_threads) : "memory");
+            asm volatile("barrier.arrive 1, %0;" ::"r"(pair_threads) : "memory");
         }
         if (!dcar) return;
         dd_add_prod(d.x, d.y, c.x, c.y, 1.0);
@@ -681,7 +684,7 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
                     av = fma(bot ? sj : f64_flip(sj, 0x80000000), bot ? yt : yb, ccj * (bot ? yb : yt));
                 }
                 if constexpr (kAuxDiag) {
-                    asm volatile("bar.sync 1, %0;" ::"r"(pair_threads) : "memory");
+                    asm volatile("barrier.sync 1, %0;" ::"r"(pair_threads) : "memory");
                     if (mine) {
                         ad = pr_ad[ce];
                         d = pr_d[ce];
