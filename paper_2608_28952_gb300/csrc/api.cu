@@ -3,7 +3,7 @@
 // A call validates its arguments, builds the pair schedule (round-robin or
 // Algorithm 3), allocates its workspace stream-ordered, and runs sweeps until
 // the stop test passes.  One sweep is a sequence of parallel steps; a step
-// launches the pivot kernel (all 2b x 2b solves of the step, one CTA per pair)
+// launches the pivot kernel (all 2b x 2b solves of the step, a CTA or a cluster per pair)
 // and the update kernel (all block-row/column updates of the step, Algorithm
 // 2).  A sweep's launches are captured once into a CUDA graph and replayed;
 // the only device->host traffic per sweep is the stop statistic.
@@ -124,8 +124,8 @@ static cudaError_t launch_step(EvdState& E, int s, int cur, cudaStream_t cs, dou
     // until the next pivots have had 4 us to start: begun any sooner, and even
     // at the same moment, it fills every SM, and a cluster waits for SMs that
     // are empty (n = 1000, b = 32: the pivots of a step 157 -> 257 us).  n = 1000,
-    // b = 32 127.5 -> 100 ms, b = 16 141.5 -> 108, n = 2000, b = 64 -7 %; FP64_EMU n
-    // = 1024, b = 32 92.7 -> 77.3, n = 2048, b = 64 281 -> 236, n = 4096 -10 %.
+    // b = 32 127.5 -> 100 ms, b = 16 141.6 -> 107, n = 2000, b = 64 787 -> 714; FP64_EMU
+    // n = 1024, b = 32 89 -> 78, n = 2048, b = 64 334 -> 289, n = 4096 1390 -> 1246.
     pa.alone = 1;
     SideStream& sd = *E.side;
     if (first >= 2 && ua.Qin && (e = cudaStreamWaitEvent(cs, sd.done[cur], 0)) != cudaSuccess) return e;

@@ -219,8 +219,8 @@ inline int choose_pivot_cluster(int k, int npairs)
 }
 
 // Whether the pivot solves leave SMs for a side stream's kernels, and those are
-// worth the events (n = 256: 12.64 ms without, 12.8 with them; n = 500: 33.3 and
-// 31.4).
+// worth the events (n = 256: 12.64 ms without, 12.8 with them; n = 500: 31.0 and
+// 29.1).
 inline bool sms_left(int np, int npairs, int pcl)
 {
     int dev = 0, sms = 0;

@@ -35,7 +35,17 @@
 //     parameters to every CTA and (t, a_pq) to whoever carries the two diagonal
 //     entries next.  Where auxiliary warps carry the diagonal they also hand
 //     over d = aqq - app and its leading bits, ready before the entry is:
-//     14 FP64 instructions are left in the chain (k = 32: 77.5 -> 69.7 us).
+//     14 FP64 instructions are left in the chain (k = 32, with shears for
+//     rotations: 77.5 -> 69.7 us a launch; 72 with rot2).
+// What ends a round (clock stamps, cycles from its start; FP64 V but where said):
+//   k, CTAs        quads stored   V done   entry formed   choice sent   round
+//   32, 1          1665           3360     925            3310          3550
+//   64, 4          1630           3380     920            3490          4240
+//   128, 6         6270           7340     2410           6730          8790
+//   128, 6, FP32   4020           3730     790            4270          5050
+// So at k <= 64 the bulk warps (quads, then V) and the chain (its choice takes
+// 2300 to 2600 cycles beside them, 14 x 64 of them FP64 issue) end together; above,
+// the FP64 unit, and the slowest CTA's share of it, decides.
 // One cluster barrier per round ("round g is stored, round g + 1's parameters
 // are there") with two buffers of the quads; where shared memory holds only
 // one, a second one ("every quad of round g is in registers") whose wait is
@@ -188,8 +198,8 @@ __global__ void __launch_bounds__(NB + CH + AT, 1) k_pivot_pos(PivotArgs a, int 
     // The auxiliary threads rotate V: an FP32 one always; an FP64 one (as much work as the quads)
     // where the FP64 unit bounds the round, not where the rotation choice does
     // and would wait behind four more FP64 warps (one quad per bulk thread;
-    // measured: k = 32 78 us with V after the quads, 82 us beside them; k = 128
-    // with 16 pairs 613 and 520 us)
+    // measured: k = 32 72 us with V after the quads, 85 us beside them; k = 128
+    // with 16 pairs 695 and 602 us)
     constexpr bool kAuxV = AT > 0 && (V32 || QPT > 1);
     // and carry the diagonal, unless an FP64 V keeps them busy (then the first
     // bulk threads do, and the chain reads its part of the diagonal itself)
@@ -898,11 +908,11 @@ bool pivot_pos_fits(int k, int C, size_t smem_cap)
 // clusters only, so npairs * C <= SMs is not enough) and that still pays, or 1.
 // A round's FP64 work per CTA shrinks with C while the rotation choice and the
 // cluster barrier do not.  Measured on GB300, us per launch with C = 1 / 2 / 4
-// / 8: k = 32 (n = 256) 78 / 82 / 84 / 78; k = 40 (n = 300) 160 / 109 / 102 /
-// 102; k = 64 (n = 512) 326 / 211 / 164 / 160; k = 96 (n = 400) 949 / 843 /
-// 441 / 310; k = 128 (n = 512) 2078 / 1510 / 756 / 425; with two waves of
-// clusters (16 pairs of C = 8) 848 instead of 767 at k = 128, 310 instead of
-// 166 at k = 64.
+// / 8: k = 32 (8 pairs) 72 / 78 / 79 / -; k = 40 132 / 99 / 96 / -; k = 64 369 / 218 /
+// 158 / 150; k = 96 (5 pairs) 1135 / 660 / 426 / 291; k = 128 (4 pairs) 2490 / 1317 /
+// 763 / 447, with 6 CTAs 600, 12 422, 16 338.  Two waves of larger clusters lose:
+// 16 pairs at k = 64 291 with 8 CTAs, at k = 128 888 with 8 and 602 with 6; 32
+// pairs at k = 256 8112 with 8 and 5138 with 4.
 int pivot_cluster_size(int k, int npairs, size_t smem_cap)
 {
     const int cmax = k <= 32 ? 1 : (k <= 64 ? 4 : (k <= 96 ? 8 : PP_MAXC));
