@@ -173,12 +173,11 @@ typedef struct {
     double off_hist[64];     /* per sweep                                      */
     double ms_total;         /* device time of the call (CUDA events)          */
     double ms_pivot;         /* device time in the pivot-solve kernels         */
-    double ms_update;        /* device time in the update kernels (A and Q /
-                                G and V; for the SVD including the Gram).  Q's
-                                and V's updates may run beside the pivot solves
-                                on a stream of their own: they count here all
-                                the same, so the two can add up to more than
-                                ms_total                                       */
+    double ms_update;        /* device time during which update kernels ran
+                                (A and Q / G and V; for the SVD including the
+                                Gram).  Q's and V's updates may run beside the
+                                pivot solves, and that time counts in both: the
+                                two can add up to more than ms_total           */
     long long launches;      /* kernels this call launched (the kernels of one
                                 emulated update count as one)                  */
     long long pivot_launches;  /* of which pivot-solve kernels                 */

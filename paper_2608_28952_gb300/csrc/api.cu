@@ -213,11 +213,16 @@ SweepResult run_evd_sweeps(EvdState& E, const jacobi_params& p, int& cur, double
             cudaStreamSynchronize(s) != cudaSuccess)
             return {JACOBI_ERR_CUDA, sw};
         st->steps += E.ord.S;
+        Spans upd;
+        float end = 0.f;
         for (int si = 0; si < E.ord.S; ++si) {
-            st->ms_pivot += pe.ms(2 * si, 2 * si + 1);
-            st->ms_update += pe.ms(2 * si + 1, 2 * si + 2);
+            const float mid = pe.at(2 * si + 1);
+            st->ms_pivot += mid - end;
+            end = pe.at(2 * si + 2);
+            upd.emplace_back(mid, end);
         }
-        st->ms_update += times.ms();
+        times.add(upd, pe.ev[0]);
+        st->ms_update += covered_ms(upd);
         // on a side stream Q's updates are launches of their own, with a pause before all but the last
         const int q_own = E.side && E.Qw[0] ? E.ord.S : 0;
         st->launches += 2 * E.ord.S + 1 + (q_own ? 2 * q_own - 1 : 0);
@@ -569,11 +574,17 @@ static int gesvd_fp64(int m, int n, double* G, int ldg, double* sigma, double* V
                 cudaStreamSynchronize(s) != cudaSuccess)
                 return JACOBI_ERR_CUDA;
             st->steps += ord.S;
+            Spans upd;
+            float end = 0.f;
             for (int si = 0; si < ord.S; ++si) {
-                st->ms_update += pe.ms(3 * si, 3 * si + 1) + pe.ms(3 * si + 2, 3 * si + 3);
-                st->ms_pivot += pe.ms(3 * si + 1, 3 * si + 2);
+                const float gram = pe.at(3 * si + 1), piv = pe.at(3 * si + 2);
+                upd.emplace_back(end, gram);
+                st->ms_pivot += piv - gram;
+                end = pe.at(3 * si + 3);
+                upd.emplace_back(piv, end);
             }
-            st->ms_update += times.ms();
+            times.add(upd, pe.ev[0]);
+            st->ms_update += covered_ms(upd);
             // on a side stream V's updates are launches of their own, with a pause before all but the last
             st->launches += 4 * ord.S + (beside ? 2 * ord.S - 1 : 0);
             st->pivot_launches += ord.S;

@@ -7,6 +7,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -83,6 +85,16 @@ struct Timer {
     }
 };
 
+inline float elapsed_ms(cudaEvent_t a, cudaEvent_t b)
+{
+    float t = 0.f;
+    if (cudaEventElapsedTime(&t, a, b) != cudaSuccess) {
+        cudaGetLastError();
+        return 0.f;
+    }
+    return t;
+}
+
 // Events recorded between the kernels of a sweep (inside the captured graph),
 // read after the sweep to split the device time into pivot and update phases.
 struct PhaseEvents {
@@ -96,19 +108,27 @@ struct PhaseEvents {
         for (auto& e : ev)
             if (e) cudaEventDestroy(e);
     }
-    float ms(size_t a, size_t b) const
-    {
-        float t = 0.f;
-        if (cudaEventElapsedTime(&t, ev[a], ev[b]) != cudaSuccess) {
-            cudaGetLastError();
-            return 0.f;
-        }
-        return t;
-    }
+    float ms(size_t a, size_t b) const { return elapsed_ms(ev[a], ev[b]); }
+    float at(size_t i) const { return i ? ms(0, i) : 0.f; }   // from the first
 };
 
-// Intervals on a side stream (its update kernels), by number; those that a sweep
-// did not open count nothing.
+// Spans of device time, in ms from a sweep's first event, and the time that any of
+// them covers (update kernels of two streams can run at the same time).
+using Spans = std::vector<std::pair<float, float>>;
+inline double covered_ms(Spans& v)
+{
+    std::sort(v.begin(), v.end());
+    double t = 0.0;
+    float end = 0.f;
+    for (const auto& x : v) {
+        t += std::max(0.f, x.second - std::max(x.first, end));
+        end = std::max(end, x.second);
+    }
+    return t;
+}
+
+// The spans of a side stream's update kernels, by number; those that a sweep did
+// not open are left out.
 struct SideTimes {
     PhaseEvents pe;
     std::vector<char> on;
@@ -119,12 +139,10 @@ struct SideTimes {
         return cudaEventRecordWithFlags(pe.ev[2 * i], s, cudaEventRecordExternal);
     }
     cudaError_t close(size_t i, cudaStream_t s) { return cudaEventRecordWithFlags(pe.ev[2 * i + 1], s, cudaEventRecordExternal); }
-    double ms() const
+    void add(Spans& v, cudaEvent_t base) const
     {
-        double t = 0.0;
         for (size_t i = 0; i < on.size(); ++i)
-            if (on[i]) t += pe.ms(2 * i, 2 * i + 1);
-        return t;
+            if (on[i]) v.emplace_back(elapsed_ms(base, pe.ev[2 * i]), elapsed_ms(base, pe.ev[2 * i + 1]));
     }
 };
 

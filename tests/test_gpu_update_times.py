@@ -49,3 +49,16 @@ def test_svd(jg):
     assert st.update_launches == 3 * S * st.sweeps and st.pivot_launches == S * st.sweeps
     assert st.launches == (6 * S - 1) * st.sweeps + 4
     assert st.flops_update / st.ms_update / 1e9 <= bench.FP64_PEAK_TFLOPS, st
+
+
+@pytest.mark.parametrize("n,b,emu", [(1536, 64, False), (2048, 64, True)])
+def test_update_time_within_the_call(jg, n, b, emu):
+    """Q's and A's updates that run at the same time count it once: the updates' time
+    is no more than the call's."""
+    import torch
+    M = torch.randn((n, n), generator=torch.Generator().manual_seed(n), dtype=torch.float64)
+    A = (0.5 * (M + M.t())).cuda()
+    kw = dict(b=b, **(dict(precision=jg.PREC_FP64_EMU) if emu else {}))
+    jg.syev(A.clone(), **kw)
+    st = jg.syev(A.clone(), **kw)[-1]
+    assert 0 < st.ms_update <= st.ms_total and 0 < st.ms_pivot <= st.ms_total
