@@ -215,12 +215,13 @@ struct Fork {
     cudaStream_t s;
     int used = 0;
     bool ok = true;
-    Fork(jacobi_plan* p, cudaStream_t st) : pl(p), s(st) {}
+    const bool in_turn;   // no side streams: everything on s
+    Fork(jacobi_plan* p, cudaStream_t st, bool turn) : pl(p), s(st), in_turn(turn) {}
     ~Fork() { join(); }   // also where a launch failed: the caller's stream waits for what was launched
     // a side stream (made when first wanted, kept by the plan); s when there is none left
     cudaStream_t next()
     {
-        if (!ok || used == kBatchedSides) return s;
+        if (!ok || in_turn || used == kBatchedSides) return s;
         if (!pl->ev_fork) ok = cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming) == cudaSuccess;
         if (ok && used == 0) ok = cudaEventRecord(pl->ev_fork, s) == cudaSuccess;
         if (ok && !pl->side[used]) {
@@ -245,10 +246,12 @@ struct Fork {
 // Launch the batch (or the sub-list `h_list` / `d_list`, matrix indices in
 // longest-first order): EVD matrices above the shared-memory size go to the
 // cluster kernel (grouped by cluster size, largest first), the rest to the
-// persistent kernel.
+// persistent kernel.  in_turn: the groups one after the other, one CTA per
+// matrix in the blocked method (what a candidate shape costs a batch that fills
+// the GPU; see jacobi_plan_autotune).
 template <typename T>
 cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape& sh, int grid,
-                        const std::vector<int>& h_list, const int* d_list)
+                        const std::vector<int>& h_list, const int* d_list, bool in_turn)
 {
     cudaError_t e = cudaMemsetAsync(pl->d_queue, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
@@ -257,7 +260,7 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
         // The groups below are independent: each goes to a stream of its own (the
         // largest orders on the one with the highest priority), so that one group's last matrices
         // do not leave the GPU idle before the next group starts.
-        Fork fork(pl, s);
+        Fork fork(pl, s, in_turn);
         BatchedEvdArgs<T> a{};
         a.n = pl->d_n;
         a.A = (T* const*)pl->d_ptrs;
@@ -291,7 +294,7 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
                 ++nb;
             }
             if (nb > 0 && (e = launch_batched_evd_blocked<T>(a, d_list, nb, pl->d_queue + 1, (T*)pl->d_blk, pl->blk_slot,
-                                                             pl->blk_grid, blk_cluster<T>(pl, h_list, nb), fork.next())) !=
+                                                             pl->blk_grid, in_turn ? 1 : blk_cluster<T>(pl, h_list, nb), fork.next())) !=
                               cudaSuccess)
                 return e;
             nl = nb;
@@ -366,10 +369,10 @@ cudaError_t plan_launch(jacobi_plan* pl, int* info, cudaStream_t s, const Shape&
 }
 
 cudaError_t plan_launch_any(jacobi_plan* pl, int* info, cudaStream_t s, const Shape& sh, int grid,
-                            const std::vector<int>& h_list, const int* d_list)
+                            const std::vector<int>& h_list, const int* d_list, bool in_turn = false)
 {
-    return pl->esize == 8 ? plan_launch<double>(pl, info, s, sh, grid, h_list, d_list)
-                          : plan_launch<float>(pl, info, s, sh, grid, h_list, d_list);
+    return pl->esize == 8 ? plan_launch<double>(pl, info, s, sh, grid, h_list, d_list, in_turn)
+                          : plan_launch<float>(pl, info, s, sh, grid, h_list, d_list, in_turn);
 }
 
 template <typename T>
@@ -526,7 +529,15 @@ extern "C" int jacobi_plan_autotune(jacobi_plan* pl, void* const* A_or_G, void* 
     }
     if (cudaMemcpyAsync(pl->d_ptrs, pl->h_ptrs, sizeof(void*) * 3 * B, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return JACOBI_ERR_CUDA;
+    // In FP64 a sample of a larger batch is timed group after group: side by side and
+    // split over clusters, as a batch of its size would run, it lasts as long as its
+    // longest matrix whatever the shape, and the choice was noise (2500 matrices of
+    // order 8..512: 6905 to 7320 ms with the shapes picked, 6909 with the one that is
+    // picked now every time).  In FP32 the sample side by side picks the better one (8000
+    // matrices: 1259 ms, 1272 with the choice group after group).  A batch that is its
+    // own sample is timed as it will run.
     const int sample = std::min(B, device_sms() * 2);
+    const bool in_turn = sample < B && pl->esize == 8;
     std::vector<int> h_sub(sample);
     for (int i = 0; i < sample; ++i) h_sub[i] = pl->h_order[(size_t)i * B / sample];
     int* d_sub = nullptr;
@@ -549,9 +560,9 @@ extern "C" int jacobi_plan_autotune(jacobi_plan* pl, void* const* A_or_G, void* 
     for (const Shape& sh : cands) {
         const int grid = std::min(grid_for(pl, sh), device_sms() * 4);
         // warm, then time
-        if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub) != cudaSuccess) { cudaGetLastError(); continue; }
+        if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub, in_turn) != cudaSuccess) { cudaGetLastError(); continue; }
         cudaEventRecord(e0, s);
-        if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub) != cudaSuccess) { cudaGetLastError(); continue; }
+        if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub, in_turn) != cudaSuccess) { cudaGetLastError(); continue; }
         cudaEventRecord(e1, s);
         if (cudaEventSynchronize(e1) != cudaSuccess) { rc = JACOBI_ERR_CUDA; break; }
         float ms = 0.f;
@@ -565,9 +576,9 @@ extern "C" int jacobi_plan_autotune(jacobi_plan* pl, void* const* A_or_G, void* 
             Shape sh = bestsh;
             sh.blk_min = bm;
             const int grid = std::min(grid_for(pl, sh), device_sms() * 4);
-            if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub) != cudaSuccess) { cudaGetLastError(); continue; }
+            if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub, in_turn) != cudaSuccess) { cudaGetLastError(); continue; }
             cudaEventRecord(e0, s);
-            if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub) != cudaSuccess) { cudaGetLastError(); continue; }
+            if (plan_launch_any(pl, info, s, sh, grid, h_sub, d_sub, in_turn) != cudaSuccess) { cudaGetLastError(); continue; }
             cudaEventRecord(e1, s);
             if (cudaEventSynchronize(e1) != cudaSuccess) { rc = JACOBI_ERR_CUDA; break; }
             float ms = 0.f;
